@@ -315,51 +315,144 @@ __global__ void entry_to_half_kernel(const float *__restrict__ p, __half *__rest
 }
 
 // ---- training (f32 master weights) on a chunk of B samples ----
-// Z[b][j] = b1[j] + sum_i W1[i][j] (s X[b][i]); 4 samples of 64 units per block
-__global__ void train_hidden_kernel(const float *__restrict__ P, const float *__restrict__ X,
-                                    int B, int d, float *__restrict__ Z, EntryLayout L) {
-    const int b = blockIdx.x * 4 + (threadIdx.x >> 6), j = threadIdx.x & 63;
-    if (b >= B)
-        return;
-    const float s = P[0];
-    float z = P[L.oB1 + j];
-    for (int i = 0; i < d; ++i)
-        z = fmaf(P[L.oW1 + (int64_t)i * EH + j], s * X[(int64_t)b * d + i], z);
-    Z[(int64_t)b * EH + j] = z;
+// The five contractions of a step run on one 64 x 64 register-tiled product (4 x 4 values
+// per thread, 32-deep chunks staged in shared memory, the next chunk's global loads in
+// flight while the current one is multiplied).  At 16,384 samples, d = 128 and E = 256 a
+// step is 2.1 GFLOP over 16 MB that stays in L2, so what counts is how many CTAs a
+// contraction fills: the outputs over samples give 256 and 1,024 tiles, and the weight
+// gradients (4 and 2 tiles of outputs) split the samples into slices of SLICE, each
+// writing its own partial sums, which grad_reduce_kernel adds in slice order (no atomics:
+// the gradient is the same in every run).  That step took 2,804 us with one thread per
+// output walking all samples of a 2,048-sample chunk in eight chunks, and takes 254 us.
+constexpr int GT = 64, GK = 32, GP = GT + 1;
+constexpr int SLICE = 128;
+
+// acc[i][j] (+)= sum over k in [k0, k1) of a(k, ty * 4 + i) b(k, tx * 4 + j), k ascending.
+// AK / BK: the operand is contiguous along k in memory (the staging loop follows it).
+template <bool AK, bool BK, class LA, class LB>
+__device__ __forceinline__ void tile_product(float acc[4][4], int64_t k0, int64_t k1, LA la, LB lb,
+                                             float (*As)[GP], float (*Bs)[GP]) {
+    const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
+    float ra[8], rb[8];
+    auto fetch = [&](int64_t kb) {
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            const int e = tid + 256 * i;
+            const int ka = AK ? e & 31 : e >> 6, r = AK ? e >> 5 : e & 63;
+            const int kk = BK ? e & 31 : e >> 6, c = BK ? e >> 5 : e & 63;
+            ra[i] = kb + ka < k1 ? la(kb + ka, r) : 0.f;
+            rb[i] = kb + kk < k1 ? lb(kb + kk, c) : 0.f;
+        }
+    };
+    fetch(k0);
+    for (int64_t kb = k0; kb < k1; kb += GK) {
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            const int e = tid + 256 * i;
+            As[AK ? e & 31 : e >> 6][AK ? e >> 5 : e & 63] = ra[i];
+            Bs[BK ? e & 31 : e >> 6][BK ? e >> 5 : e & 63] = rb[i];
+        }
+        __syncthreads();
+        if (kb + GK < k1)
+            fetch(kb + GK);
+#pragma unroll 8
+        for (int kk = 0; kk < GK; ++kk) {
+            float a[4], b[4];
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                a[i] = As[kk][ty * 4 + i];
+                b[i] = Bs[kk][tx + 16 * i];
+            }
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+#pragma unroll
+                for (int j = 0; j < 4; ++j)
+                    acc[i][j] = fmaf(a[i], b[j], acc[i][j]);
+        }
+        __syncthreads();
+    }
 }
 
-// Tl[b][o] = b2[o] + sum_h W2[h][o] relu(Z[b][h]); grid (ceil(E/128), B)
-__global__ void train_out_kernel(const float *__restrict__ P, const float *__restrict__ Z, int E,
-                                 float *__restrict__ Tl, EntryLayout L) {
-    __shared__ float h[EH];
-    const int b = blockIdx.y;
-    if (threadIdx.x < EH)
-        h[threadIdx.x] = fmaxf(Z[(int64_t)b * EH + threadIdx.x], 0.f);
-    __syncthreads();
-    const int o = blockIdx.x * blockDim.x + threadIdx.x;
-    if (o >= E)
-        return;
-    float t = P[L.oB2 + o];
-    for (int k = 0; k < EH; ++k)
-        t = fmaf(P[L.oW2 + (int64_t)k * E + o], h[k], t);
-    Tl[(int64_t)b * E + o] = t;
+// H[b][j] = relu(b1[j] + sum_i W1[i][j] (s X[b][i])), i ascending; grid (ceil(B/64))
+__global__ void __launch_bounds__(256) train_hidden_kernel(const float *__restrict__ P,
+                                                           const float *__restrict__ X, int B,
+                                                           int d, float *__restrict__ H,
+                                                           EntryLayout L) {
+    __shared__ float As[GK][GP], Bs[GK][GP];
+    const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
+    const int b0 = blockIdx.x * GT;
+    const float s = P[0];
+    float acc[4][4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+        const float bias = P[L.oB1 + tx + 16 * j];
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+            acc[i][j] = bias;
+    }
+    tile_product<true, false>(
+        acc, 0, d,
+        [&](int64_t k, int r) { return b0 + r < B ? s * X[(int64_t)(b0 + r) * d + k] : 0.f; },
+        [&](int64_t k, int c) { return P[L.oW1 + k * EH + c]; }, As, Bs);
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        const int b = b0 + ty * 4 + i;
+        if (b >= B)
+            continue;
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+            H[(int64_t)b * EH + tx + 16 * j] = fmaxf(acc[i][j], 0.f);
+    }
+}
+
+// T[b][o] = b2[o] + sum_h W2[h][o] H[b][h], h ascending; grid (ceil(B/64), ceil(E/64))
+__global__ void __launch_bounds__(256) train_out_kernel(const float *__restrict__ P,
+                                                        const float *__restrict__ H, int B, int E,
+                                                        float *__restrict__ T, EntryLayout L) {
+    __shared__ float As[GK][GP], Bs[GK][GP];
+    const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
+    const int b0 = blockIdx.x * GT, o0 = blockIdx.y * GT;
+    float acc[4][4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+        const int o = o0 + tx + 16 * j;
+        const float bias = o < E ? P[L.oB2 + o] : 0.f;
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+            acc[i][j] = bias;
+    }
+    tile_product<true, false>(
+        acc, 0, EH,
+        [&](int64_t k, int r) { return b0 + r < B ? H[(int64_t)(b0 + r) * EH + k] : 0.f; },
+        [&](int64_t k, int c) { return o0 + c < E ? P[L.oW2 + k * E + o0 + c] : 0.f; }, As, Bs);
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        const int b = b0 + ty * 4 + i;
+        if (b >= B)
+            continue;
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            const int o = o0 + tx + 16 * j;
+            if (o < E)
+                T[(int64_t)b * E + o] = acc[i][j];
+        }
+    }
 }
 
 // dT = (softmax(T) - onehot(label)) * inv_n per sample (a warp each); loss += (lse - t_y) * inv_n.
 // A label outside 0..E-1 contributes nothing.
-__global__ void train_softmax_kernel(const float *__restrict__ Tl, const int32_t *__restrict__ y,
-                                     int B, int E, float inv_n, float *__restrict__ dT,
-                                     float *__restrict__ loss) {
+// T becomes dT in place (a lane reads the elements that it writes).
+__global__ void train_softmax_kernel(float *T, const int32_t *__restrict__ y, int B, int E,
+                                     float inv_n, float *__restrict__ loss) {
     const int lane = threadIdx.x & 31;
     const int b = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
     if (b >= B)
         return;
-    const float *t = Tl + (int64_t)b * E;
-    float *g = dT + (int64_t)b * E;
+    float *t = T + (int64_t)b * E;
     const int lab = y[b];
     if (lab < 0 || lab >= E) {
         for (int o = lane; o < E; o += 32)
-            g[o] = 0.f;
+            t[o] = 0.f;
         return;
     }
     float mx = -INFINITY;
@@ -375,66 +468,90 @@ __global__ void train_softmax_kernel(const float *__restrict__ Tl, const int32_t
     for (int o = 16; o > 0; o >>= 1)
         se += __shfl_xor_sync(FULL, se, o);
     const float lse = mx + logf(se);
-    for (int o = lane; o < E; o += 32)
-        g[o] = (expf(t[o] - lse) - (o == lab ? 1.f : 0.f)) * inv_n;
     if (lane == 0)
         atomicAdd(loss, (lse - t[lab]) * inv_n);
-}
-
-// G[W2][h][o] += sum_b relu(Z[b][h]) dT[b][o]; row h = 64 is b2 (sum_b dT[b][o])
-__global__ void train_gw2_kernel(const float *__restrict__ Z, const float *__restrict__ dT, int B,
-                                 int E, float *__restrict__ G, EntryLayout L) {
-    const int h = blockIdx.y;
-    const int o = blockIdx.x * blockDim.x + threadIdx.x;
-    if (o >= E)
-        return;
-    float acc = 0.f;
-    for (int b = 0; b < B; ++b) {
-        const float hv = h < EH ? fmaxf(Z[(int64_t)b * EH + h], 0.f) : 1.f;
-        acc = fmaf(hv, dT[(int64_t)b * E + o], acc);
-    }
-    if (h < EH)
-        G[L.oW2 + (int64_t)h * E + o] += acc;
-    else
-        G[L.oB2 + o] += acc;
-}
-
-// dZ[b][h] = [Z > 0] sum_o dT[b][o] W2[h][o]; a warp per (b, h) pair group of 1
-__global__ void train_dz_kernel(const float *__restrict__ P, const float *__restrict__ Z,
-                                const float *__restrict__ dT, int B, int E,
-                                float *__restrict__ dZ, EntryLayout L) {
-    const int lane = threadIdx.x & 31;
-    const int64_t pair = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-    if (pair >= (int64_t)B * EH)
-        return;
-    const int b = (int)(pair / EH), h = (int)(pair % EH);
-    float acc = 0.f;
+    __syncwarp();  // the label's logit is read before its lane overwrites it
     for (int o = lane; o < E; o += 32)
-        acc = fmaf(dT[(int64_t)b * E + o], P[L.oW2 + (int64_t)h * E + o], acc);
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1)
-        acc += __shfl_xor_sync(FULL, acc, o);
-    if (lane == 0)
-        dZ[(int64_t)b * EH + h] = Z[(int64_t)b * EH + h] > 0.f ? acc : 0.f;
+        t[o] = (expf(t[o] - lse) - (o == lab ? 1.f : 0.f)) * inv_n;
 }
 
-// G[W1][i][h] += sum_b s X[b][i] dZ[b][h]; row i = d is b1 (sum_b dZ[b][h]); 4 rows of 64
-__global__ void train_gw1_kernel(const float *__restrict__ P, const float *__restrict__ X,
-                                 const float *__restrict__ dZ, int B, int d,
-                                 float *__restrict__ G, EntryLayout L) {
-    const int i = blockIdx.x * 4 + (threadIdx.x >> 6), h = threadIdx.x & 63;
-    if (i > d)
-        return;
-    const float s = P[0];
-    float acc = 0.f;
-    for (int b = 0; b < B; ++b) {
-        const float x = i < d ? s * X[(int64_t)b * d + i] : 1.f;
-        acc = fmaf(x, dZ[(int64_t)b * EH + h], acc);
+// dZ[b][h] = [H > 0] sum_o dT[b][o] W2[h][o], o ascending; grid (ceil(B/64))
+__global__ void __launch_bounds__(256) train_dz_kernel(const float *__restrict__ P,
+                                                       const float *__restrict__ H,
+                                                       const float *__restrict__ dT, int B, int E,
+                                                       float *__restrict__ dZ, EntryLayout L) {
+    __shared__ float As[GK][GP], Bs[GK][GP];
+    const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
+    const int b0 = blockIdx.x * GT;
+    float acc[4][4] = {};
+    tile_product<true, true>(
+        acc, 0, E,
+        [&](int64_t k, int r) { return b0 + r < B ? dT[(int64_t)(b0 + r) * E + k] : 0.f; },
+        [&](int64_t k, int c) { return P[L.oW2 + (int64_t)c * E + k]; }, As, Bs);
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        const int b = b0 + ty * 4 + i;
+        if (b >= B)
+            continue;
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            const int64_t e = (int64_t)b * EH + tx + 16 * j;
+            dZ[e] = H[e] > 0.f ? acc[i][j] : 0.f;
+        }
     }
-    if (i < d)
-        G[L.oW1 + (int64_t)i * EH + h] += acc;
-    else
-        G[L.oB1 + h] += acc;
+}
+
+// Partial sums of one weight gradient over a slice of samples: part[slice][r][c] =
+// sum_b A[b][r] D[b][c] for r < rows (times the input scale when scale is set) and row
+// r = rows the plain sums of D (the bias).  A has rows values per sample, D cols;
+// grid (ceil(cols/64), ceil((rows+1)/64), slices).
+__global__ void __launch_bounds__(256) train_gw_kernel(const float *__restrict__ A, int rows,
+                                                       const float *__restrict__ scale,
+                                                       const float *__restrict__ D, int cols,
+                                                       int B, float *__restrict__ part) {
+    __shared__ float As[GK][GP], Bs[GK][GP];
+    const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
+    const int c0 = blockIdx.x * GT, r0 = blockIdx.y * GT;
+    const int64_t b0 = (int64_t)blockIdx.z * SLICE;
+    const int64_t b1 = b0 + SLICE < B ? b0 + SLICE : B;
+    const float s = scale != nullptr ? *scale : 1.f;
+    float acc[4][4] = {};
+    tile_product<false, false>(
+        acc, b0, b1,
+        [&](int64_t k, int r) {
+            return r0 + r < rows ? s * A[k * rows + r0 + r] : r0 + r == rows ? 1.f : 0.f;
+        },
+        [&](int64_t k, int c) { return c0 + c < cols ? D[k * cols + c0 + c] : 0.f; }, As, Bs);
+    float *out = part + (int64_t)blockIdx.z * (rows + 1) * cols;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        const int r = r0 + ty * 4 + i;
+        if (r > rows)
+            continue;
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            const int c = c0 + tx + 16 * j;
+            if (c < cols)
+                out[(int64_t)r * cols + c] = acc[i][j];
+        }
+    }
+}
+
+// G += the slices of both gradients, in slice order.  W1 | b1 and W2 | b2 are each one
+// run of the parameter vector, laid out as train_gw_kernel lays out its rows.
+__global__ void grad_reduce_kernel(const float *__restrict__ part1, int64_t n1,
+                                   const float *__restrict__ part2, int64_t n2, int slices,
+                                   float *__restrict__ G) {
+    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n1 + n2;
+         i += (int64_t)gridDim.x * blockDim.x) {
+        const float *p = i < n1 ? part1 + i : part2 + (i - n1);
+        const int64_t step = i < n1 ? n1 : n2;
+        float acc = 0.f;
+#pragma unroll 8
+        for (int z = 0; z < slices; ++z)
+            acc += p[z * step];
+        G[1 + i] += acc;
+    }
 }
 
 // Adam (beta1 0.9, beta2 0.999) on every parameter but the input scale (index 0)
@@ -570,9 +687,22 @@ cudaError_t launch_entry_labels(const uint32_t *ids, int k, int64_t n, const uin
     return cudaGetLastError();
 }
 
-// Working memory of one chunk of B samples: Z, dZ [B][64], Tl, dT [B][E].
-size_t entry_train_chunk_bytes(int B, int E) {
-    return sizeof(float) * ((size_t)B * EH * 2 + (size_t)B * E * 2) + 1024;
+// Samples of one gradient pass: as many as keep a chunk's working memory at about 32 MB
+// (it then stays in L2 between the kernels), in whole slices and at least 2,048.
+int entry_train_chunk(int64_t n, int d, int E) {
+    const int64_t per = 2 * EH + E + ((int64_t)(d + 1) * EH + (int64_t)(EH + 1) * E) / SLICE + 1;
+    int64_t B = (int64_t(8) << 20) / per / SLICE * SLICE;
+    B = B < 2048 ? 2048 : B > 65536 ? 65536 : B;
+    return (int)(n < B ? n : B);
+}
+
+// Working memory of one chunk of B samples: H, dZ [B][64], T [B][E] and the slices' partial
+// sums of (W1 | b1) and (W2 | b2).
+size_t entry_train_chunk_bytes(int B, int d, int E) {
+    const size_t slices = ((size_t)B + SLICE - 1) / SLICE;
+    return sizeof(float) * ((size_t)B * EH * 2 + (size_t)B * E +
+                            slices * ((size_t)(d + 1) * EH + (size_t)(EH + 1) * E)) +
+           1024;
 }
 
 // Adds the gradient of the loss over samples [0, n) (divided by `total`) to G and the loss
@@ -581,22 +711,30 @@ cudaError_t entry_grad_accumulate(const float *P, int d, int E, const float *X,
                                   const int32_t *y, int64_t n, int64_t total, int B, float *G,
                                   float *loss, void *work, cudaStream_t s) {
     const EntryLayout L = entry_layout(d, E);
-    float *Z = reinterpret_cast<float *>(work);
-    float *dZ = Z + (size_t)B * EH;
-    float *Tl = dZ + (size_t)B * EH;
-    float *dT = Tl + (size_t)B * E;
+    const int64_t n1 = (int64_t)(d + 1) * EH, n2 = (int64_t)(EH + 1) * E;
+    float *H = reinterpret_cast<float *>(work);
+    float *dZ = H + (size_t)B * EH;
+    float *T = dZ + (size_t)B * EH;
+    float *part1 = T + (size_t)B * E;
+    float *part2 = part1 + (size_t)((B + SLICE - 1) / SLICE) * n1;
     const float inv = 1.f / (float)total;
+    const unsigned et = (unsigned)((E + GT - 1) / GT);
     cudaError_t e = cudaSuccess;
     for (int64_t b0 = 0; b0 < n; b0 += B) {
         const int nb = (int)(n - b0 < B ? n - b0 : B);
         const float *Xb = X + b0 * d;
-        train_hidden_kernel<<<(nb + 3) / 4, 256, 0, s>>>(P, Xb, nb, d, Z, L);
-        train_out_kernel<<<dim3((E + 127) / 128, nb), 128, 0, s>>>(P, Z, E, Tl, L);
-        train_softmax_kernel<<<(nb + 7) / 8, 256, 0, s>>>(Tl, y + b0, nb, E, inv, dT, loss);
-        train_gw2_kernel<<<dim3((E + 127) / 128, EH + 1), 128, 0, s>>>(Z, dT, nb, E, G, L);
-        train_dz_kernel<<<(unsigned)(((int64_t)nb * EH + 7) / 8), 256, 0, s>>>(P, Z, dT, nb, E,
-                                                                               dZ, L);
-        train_gw1_kernel<<<(d + 1 + 3) / 4, 256, 0, s>>>(P, Xb, dZ, nb, d, G, L);
+        const unsigned bt = (unsigned)((nb + GT - 1) / GT);
+        const unsigned sl = (unsigned)((nb + SLICE - 1) / SLICE);
+        train_hidden_kernel<<<bt, 256, 0, s>>>(P, Xb, nb, d, H, L);
+        train_out_kernel<<<dim3(bt, et), 256, 0, s>>>(P, H, nb, E, T, L);
+        train_softmax_kernel<<<(nb + 7) / 8, 256, 0, s>>>(T, y + b0, nb, E, inv, loss);
+        train_gw_kernel<<<dim3(et, (EH + GT) / GT, sl), 256, 0, s>>>(H, EH, nullptr, T, E, nb,
+                                                                    part2);
+        train_dz_kernel<<<bt, 256, 0, s>>>(P, H, T, nb, E, dZ, L);
+        train_gw_kernel<<<dim3(1, (unsigned)((d + GT) / GT), sl), 256, 0, s>>>(Xb, d, P, dZ, EH,
+                                                                              nb, part1);
+        grad_reduce_kernel<<<grid_for(n1 + n2, 256), 256, 0, s>>>(part1, n1, part2, n2, (int)sl,
+                                                                  G);
         if ((e = cudaGetLastError()) != cudaSuccess)
             return e;
     }

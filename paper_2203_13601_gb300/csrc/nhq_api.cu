@@ -837,9 +837,9 @@ nhq_status nhq_entry_grad(const float *params, int32_t d, int32_t E, const float
     CK(cudaMemsetAsync(loss, 0, sizeof(float), s));
     if (n == 0)
         return NHQ_OK;
-    const int B = 2048;
+    const int B = entry_train_chunk(n, d, E);
     void *work = nullptr;
-    CK(cudaMallocAsync(&work, entry_train_chunk_bytes(B, E), s));
+    CK(cudaMallocAsync(&work, entry_train_chunk_bytes(B, d, E), s));
     cudaError_t e = entry_grad_accumulate(params, d, E, queries, labels, n, n, B, grad, loss,
                                           work, s);
     cudaFreeAsync(work, s);
@@ -860,11 +860,11 @@ nhq_status nhq_entry_train(float *params, int32_t d, int32_t E, const float *que
         return NHQ_OK;
     cudaStream_t s = as_stream(stream);
     const int64_t np = entry_param_count(d, E);
-    const int B = batch < 2048 ? batch : 2048;  // chunk of one gradient pass
+    const int B = entry_train_chunk(n < batch ? n : batch, d, E);
     float *buf = nullptr;  // gradient, first and second moments, loss
     void *work = nullptr;
     CK(cudaMallocAsync(&buf, sizeof(float) * (size_t)(3 * np + 1), s));
-    cudaError_t e = cudaMallocAsync(&work, entry_train_chunk_bytes(B, E), s);
+    cudaError_t e = cudaMallocAsync(&work, entry_train_chunk_bytes(B, d, E), s);
     float *g = buf, *m = buf + np, *v = m + np, *loss = v + np;
     if (e == cudaSuccess)
         e = cudaMemsetAsync(m, 0, sizeof(float) * (size_t)(2 * np), s);

@@ -418,7 +418,8 @@ cudaError_t launch_entry_scores_learned(const __half *w16, const float *params, 
                                         float *hidden, float *out, cudaStream_t s);
 cudaError_t launch_entry_labels(const uint32_t *ids, int k, int64_t n, const uint32_t *cell,
                                 int64_t N, int32_t *labels, cudaStream_t s);
-size_t entry_train_chunk_bytes(int B, int E);
+int entry_train_chunk(int64_t n, int d, int E);
+size_t entry_train_chunk_bytes(int B, int d, int E);
 cudaError_t entry_grad_accumulate(const float *P, int d, int E, const float *X,
                                   const int32_t *y, int64_t n, int64_t total, int B, float *G,
                                   float *loss, void *work, cudaStream_t s);
