@@ -15,8 +15,7 @@
 // enter), accumulate squared distances with teams of 8 lanes (128-bit loads,
 // shuffle reduction), finish every candidate's Gamma in one warp-wide step
 // (lane j holds candidate j's record in a register), and merge the survivors
-// into the pool (rank by broadcast compares for up to 8, warp bitonic sort
-// beyond).
+// into the pool (the places of the merged order computed per chunk of 32 records).
 //
 // The pool after every expansion equals the serial algorithm's: inserting a
 // batch and keeping the ef smallest equals inserting the batch one record at a

@@ -55,21 +55,6 @@ __device__ __forceinline__ bool hash_contains(const uint32_t *h, int bits, uint3
     return false;
 }
 
-__device__ __forceinline__ unsigned long long warp_sort_asc(unsigned long long x, int lane) {
-#pragma unroll
-    for (int k = 2; k <= 32; k <<= 1) {
-#pragma unroll
-        for (int j = k >> 1; j > 0; j >>= 1) {
-            unsigned long long y = __shfl_xor_sync(FULL, x, j);
-            bool up = (lane & k) == 0;
-            bool lower = (lane & j) == 0;
-            unsigned long long lo = x < y ? x : y, hi = x < y ? y : x;
-            x = (lower == up) ? lo : hi;
-        }
-    }
-    return x;
-}
-
 // number of pool records whose (Gamma, id) is below key c (flag bits ignored)
 __device__ __forceinline__ int pool_lower_bound(const unsigned long long *pool, int n,
                                                 unsigned long long c) {
@@ -77,19 +62,6 @@ __device__ __forceinline__ int pool_lower_bound(const unsigned long long *pool, 
     while (lo < hi) {
         int mid = (lo + hi) >> 1;
         if ((pool[mid] & ~1ull) < c)
-            lo = mid + 1;
-        else
-            hi = mid;
-    }
-    return lo;
-}
-
-__device__ __forceinline__ int sorted_count_less(const unsigned long long *s, int n,
-                                                 unsigned long long x) {
-    int lo = 0, hi = n;
-    while (lo < hi) {
-        int mid = (lo + hi) >> 1;
-        if (s[mid] < x)
             lo = mid + 1;
         else
             hi = mid;
@@ -305,18 +277,14 @@ __device__ __forceinline__ unsigned long long warp_min_key(unsigned long long x)
     return ((unsigned long long)hi << 32) | lo;
 }
 
-// number of pool records below c, every lane passing the same c (ballot count)
+// number of pool records below c, every lane passing the same c: the whole chunks of 32
+// below it by their last records (n <= 1,024, so one ballot), then the chunk it falls into
 __device__ __forceinline__ int pool_rank_uniform(const unsigned long long *pool, int n,
                                                  unsigned long long c, int lane) {
-    int r = 0;
-    for (int b = 0; b < n; b += 32) {
-        const int i = b + lane;
-        const unsigned m = __ballot_sync(FULL, i < n && (pool[i] & ~1ull) < c);
-        r += __popc(m);
-        if (m != FULL)
-            break;  // sorted: the first record not below c ends the run
-    }
-    return r;
+    const int last = 32 * lane + 31;
+    int b = n > 32 ? 32 * __popc(__ballot_sync(FULL, last < n && (pool[last] & ~1ull) < c)) : 0;
+    const int i = b + lane;
+    return b + __popc(__ballot_sync(FULL, i < n && (pool[i] & ~1ull) < c));
 }
 
 // Drop a candidate that cannot enter: above the last record of a full pool, or,
@@ -337,71 +305,55 @@ __device__ __forceinline__ unsigned long long filter_key(unsigned long long c,
 }
 
 // Inserts the candidate records held one per lane (kInfKey = none) into the pool,
-// keeping its ef smallest records; equals inserting them one at a time.
+// keeping its ef smallest records; equals inserting them one at a time.  A candidate's
+// place in the merged order is its rank among the candidates plus its rank in the pool;
+// the places are distinct, so a chunk of 32 places is described by one mask, and a place
+// that no candidate takes receives the old record as many places below it as candidates
+// precede it.  Chunks go from the top down, each read before it is written.
+// A chunk costs about 20 instructions whatever the number of candidates (it was 15 plus 6
+// for each of up to 8, or a sort and a binary search per record beyond): 1,000 queries at
+// ef 100 on 10,000 objects 428 -> 391 us, 10,000 at ef 24 on a million 472 -> 451 us.
 __device__ void merge_round(unsigned long long *pool, int &n, int ef, unsigned long long c,
-                            unsigned long long *sorted32, int lane) {
+                            unsigned long long *cand32, int lane) {
     if (c != kInfKey && n == ef && c > (pool[ef - 1] & ~1ull))
         c = kInfKey;
-    const unsigned vb = __ballot_sync(FULL, c != kInfKey);
+    const bool valid = c != kInfKey;
+    const unsigned vb = __ballot_sync(FULL, valid);
     if (vb == 0)
         return;
     const int nv = __popc(vb);
-    if (nv <= 8) {
-        int rank = 0;
-        for (unsigned mm = vb; mm; mm &= mm - 1) {
-            const unsigned long long cj = __shfl_sync(FULL, c, __ffs(mm) - 1);
-            rank += cj < c ? 1 : 0;
+    const unsigned lt = lanemask_lt(lane);
+    cand32[valid ? __popc(vb & lt) : nv + __popc(~vb & lt)] = c;
+    __syncwarp();
+    int pos = ef;
+    if (valid) {
+        pos = pool_lower_bound(pool, n, c);
+#pragma unroll 2
+        for (int j = 0; j < nv; j += 2) {  // the slots after the nv candidates hold kInfKey
+            const ulonglong2 o = *reinterpret_cast<const ulonglong2 *>(cand32 + j);
+            pos += (o.x < c ? 1 : 0) + (o.y < c ? 1 : 0);
         }
-        const int pos = c != kInfKey ? rank + pool_lower_bound(pool, n, c) : ef;
-        const int p0 = (int)__reduce_min_sync(FULL, (unsigned)pos);
-        if (p0 < ef) {
-            for (int b = (n - 1) & ~31; n > 0 && b >= (p0 & ~31); b -= 32) {
-                const int e = b + lane;
-                const bool mv = e >= p0 && e < n;
-                const unsigned long long val = mv ? pool[e] : 0ull;
-                int sh = 0;
-                for (unsigned mm = vb; mm; mm &= mm - 1) {
-                    const unsigned long long cj = __shfl_sync(FULL, c, __ffs(mm) - 1);
-                    sh += cj < (val & ~1ull) ? 1 : 0;
-                }
-                __syncwarp();
-                if (mv && e + sh < ef)
-                    pool[e + sh] = val;
-                __syncwarp();
-            }
-            if (c != kInfKey && pos < ef)
-                pool[pos] = c;
-            __syncwarp();
-            n = min(ef, n + nv);
-        }
+    }
+    const int p0 = (int)__reduce_min_sync(FULL, (unsigned)pos);
+    if (p0 >= ef)
         return;
-    }
-    c = warp_sort_asc(c, lane);
-    __syncwarp();
-    sorted32[lane] = c;
-    __syncwarp();
-    const int pos = lane < nv ? lane + pool_lower_bound(pool, n, c) : ef;
-    const int p0 = __shfl_sync(FULL, pos, 0);
-    if (p0 < ef) {
-        for (int b = (n - 1) & ~31; n > 0 && b >= (p0 & ~31); b -= 32) {
-            const int e = b + lane;
-            const bool mv = e >= p0 && e < n;
-            unsigned long long val = 0;
-            int dst = ef;
-            if (mv) {
-                val = pool[e];
-                dst = e + sorted_count_less(sorted32, nv, val & ~1ull);
-            }
-            __syncwarp();
-            if (mv && dst < ef)
-                pool[dst] = val;
-            __syncwarp();
-        }
-        if (lane < nv && pos < ef)
-            pool[pos] = c;
+    const int nn = min(ef, n + nv);
+    for (int b = (nn - 1) & ~31; b >= (p0 & ~31); b -= 32) {
+        const int p = b + lane;
+        const unsigned rel = (unsigned)(pos - b);
+        const unsigned m = __reduce_or_sync(FULL, valid && rel < 32u ? 1u << rel : 0u);
+        const int below = __popc(__ballot_sync(FULL, valid && pos < b)) + __popc(m & lt);
+        const bool mv = p >= p0 && p < nn && !((m >> lane) & 1u);
+        const unsigned long long val = mv ? pool[p - below] : 0ull;
         __syncwarp();
-        n = min(ef, n + nv);
+        if (mv)
+            pool[p] = val;
+        __syncwarp();
     }
+    if (valid && pos < ef)
+        pool[pos] = c;
+    __syncwarp();
+    n = nn;
 }
 
 // index of the first unexpanded record at or after `from`, or -1
@@ -505,7 +457,7 @@ __device__ __forceinline__ void group_eval(const VT *X, int xstride, const float
 }
 
 struct WarpLayout {
-    size_t pool, sorted, d2s, cid, cchi, hash, qv, ctl, total;
+    size_t pool, cand, d2s, cid, cchi, hash, qv, ctl, total;
 };
 
 __host__ __device__ inline WarpLayout warp_layout(int ef_cap, int hash_bits, int xstride) {
@@ -513,7 +465,7 @@ __host__ __device__ inline WarpLayout warp_layout(int ef_cap, int hash_bits, int
     size_t o = 0;
     L.pool = o;
     o += sizeof(unsigned long long) * ef_cap;
-    L.sorted = o;
+    L.cand = o;
     o += sizeof(unsigned long long) * 32;
     L.d2s = o;
     o += sizeof(float) * CAND;
@@ -551,7 +503,7 @@ __global__ void __launch_bounds__(
     const WarpLayout L = warp_layout(ef_cap, a.hash_bits, a.xstride);
     unsigned char *base = smem + grp * L.total;
     unsigned long long *pool = reinterpret_cast<unsigned long long *>(base + L.pool);
-    unsigned long long *sorted32 = reinterpret_cast<unsigned long long *>(base + L.sorted);
+    unsigned long long *cand32 = reinterpret_cast<unsigned long long *>(base + L.cand);
     float *d2s = reinterpret_cast<float *>(base + L.d2s);
     uint32_t *cid = reinterpret_cast<uint32_t *>(base + L.cid);
     int *cchi = reinterpret_cast<int *>(base + L.cchi);
@@ -632,7 +584,7 @@ __global__ void __launch_bounds__(
             if (cnt > 0) {
                 group_eval<VT, CPL, EXACT, RPT, GROUP>(Xs, a.xstride, qv, cid, d2s, cnt, lane,
                                                        wpq, grp, ctl, 0);
-                merge_round(pool, n, ef, candidate_key(lane, cnt, d2s, cid, cchi, a.w), sorted32,
+                merge_round(pool, n, ef, candidate_key(lane, cnt, d2s, cid, cchi, a.w), cand32,
                             lane);
             }
         }
@@ -664,7 +616,7 @@ __global__ void __launch_bounds__(
             if (cnt > 0) {
                 group_eval<VT, CPL, EXACT, RPT, GROUP>(Xs, a.xstride, qv, cid, d2s, cnt, lane,
                                                        wpq, grp, ctl, 0);
-                merge_round(pool, n, ef, candidate_key(lane, cnt, d2s, cid, cchi, a.w), sorted32,
+                merge_round(pool, n, ef, candidate_key(lane, cnt, d2s, cid, cchi, a.w), cand32,
                             lane);
             }
         }
@@ -825,9 +777,9 @@ __global__ void __launch_bounds__(
                 adj = load_adjacency<TWO>(a, next_id, lane);
             since_change = (cmin != kInfKey && cpos < k) ? 0 : since_change + 1;
             if (cmin != kInfKey) {
-                merge_round(pool, n, ef, k0, sorted32, lane);
+                merge_round(pool, n, ef, k0, cand32, lane);
                 if (TWO)
-                    merge_round(pool, n, ef, k1, sorted32, lane);
+                    merge_round(pool, n, ef, k1, cand32, lane);
                 cursor = min(cursor, cpos);
             }
             pidx = next;
