@@ -323,7 +323,7 @@ __global__ void entry_to_half_kernel(const float *__restrict__ p, __half *__rest
 // gradients (4 and 2 tiles of outputs) split the samples into slices of SLICE, each
 // writing its own partial sums, which grad_reduce_kernel adds in slice order (no atomics:
 // the gradient is the same in every run).  That step took 2,804 us with one thread per
-// output walking all samples of a 2,048-sample chunk in eight chunks, and takes 254 us.
+// output walking all samples of a 2,048-sample chunk in eight chunks, and takes 158 us.
 constexpr int GT = 64, GK = 32, GP = GT + 1;
 constexpr int SLICE = 128;
 
@@ -439,40 +439,50 @@ __global__ void __launch_bounds__(256) train_out_kernel(const float *__restrict_
     }
 }
 
-// dT = (softmax(T) - onehot(label)) * inv_n per sample (a warp each); loss += (lse - t_y) * inv_n.
+// dT = (softmax(T) - onehot(label)) * inv_n per sample (a warp each); loss += (lse - t_y) * inv_n
+// (one addition to it per block of eight samples).
 // A label outside 0..E-1 contributes nothing.
 // T becomes dT in place (a lane reads the elements that it writes).
 __global__ void train_softmax_kernel(float *T, const int32_t *__restrict__ y, int B, int E,
                                      float inv_n, float *__restrict__ loss) {
-    const int lane = threadIdx.x & 31;
-    const int b = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-    if (b >= B)
-        return;
+    __shared__ float part[8];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int b = blockIdx.x * 8 + warp;
+    const int lab = b < B ? y[b] : -1;
     float *t = T + (int64_t)b * E;
-    const int lab = y[b];
-    if (lab < 0 || lab >= E) {
+    float mine = 0.f;
+    if (lab >= 0 && lab < E) {
+        float mx = -INFINITY;
+        for (int o = lane; o < E; o += 32)
+            mx = fmaxf(mx, t[o]);
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1)
+            mx = fmaxf(mx, __shfl_xor_sync(FULL, mx, o));
+        float se = 0.f;
+        for (int o = lane; o < E; o += 32)
+            se += expf(t[o] - mx);
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1)
+            se += __shfl_xor_sync(FULL, se, o);
+        const float lse = mx + logf(se);
+        mine = (lse - t[lab]) * inv_n;
+        __syncwarp();  // the label's logit is read before its lane overwrites it
+        for (int o = lane; o < E; o += 32)
+            t[o] = (expf(t[o] - lse) - (o == lab ? 1.f : 0.f)) * inv_n;
+    } else if (b < B) {
         for (int o = lane; o < E; o += 32)
             t[o] = 0.f;
-        return;
     }
-    float mx = -INFINITY;
-    for (int o = lane; o < E; o += 32)
-        mx = fmaxf(mx, t[o]);
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1)
-        mx = fmaxf(mx, __shfl_xor_sync(FULL, mx, o));
-    float se = 0.f;
-    for (int o = lane; o < E; o += 32)
-        se += expf(t[o] - mx);
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1)
-        se += __shfl_xor_sync(FULL, se, o);
-    const float lse = mx + logf(se);
     if (lane == 0)
-        atomicAdd(loss, (lse - t[lab]) * inv_n);
-    __syncwarp();  // the label's logit is read before its lane overwrites it
-    for (int o = lane; o < E; o += 32)
-        t[o] = (expf(t[o] - lse) - (o == lab ? 1.f : 0.f)) * inv_n;
+        part[warp] = mine;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        float sum = 0.f;
+#pragma unroll
+        for (int w = 0; w < 8; ++w)
+            sum += part[w];
+        atomicAdd(loss, sum);
+    }
 }
 
 // dZ[b][h] = [H > 0] sum_o dT[b][o] W2[h][o], o ascending; grid (ceil(B/64))
@@ -537,20 +547,35 @@ __global__ void __launch_bounds__(256) train_gw_kernel(const float *__restrict__
     }
 }
 
-// G += the slices of both gradients, in slice order.  W1 | b1 and W2 | b2 are each one
+// G += the slices of both gradients: 32 values per block, eight warps summing every
+// eighth slice in order, then the eight sums in order.  W1 | b1 and W2 | b2 are each one
 // run of the parameter vector, laid out as train_gw_kernel lays out its rows.
-__global__ void grad_reduce_kernel(const float *__restrict__ part1, int64_t n1,
-                                   const float *__restrict__ part2, int64_t n2, int slices,
-                                   float *__restrict__ G) {
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n1 + n2;
-         i += (int64_t)gridDim.x * blockDim.x) {
-        const float *p = i < n1 ? part1 + i : part2 + (i - n1);
-        const int64_t step = i < n1 ? n1 : n2;
+__global__ void __launch_bounds__(256) grad_reduce_kernel(const float *__restrict__ part1,
+                                                          int64_t n1,
+                                                          const float *__restrict__ part2,
+                                                          int64_t n2, int slices,
+                                                          float *__restrict__ G) {
+    __shared__ float sums[8][32];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    for (int64_t i0 = blockIdx.x * (int64_t)32; i0 < n1 + n2; i0 += (int64_t)gridDim.x * 32) {
+        const int64_t i = i0 + lane;
         float acc = 0.f;
+        if (i < n1 + n2) {
+            const float *p = i < n1 ? part1 + i : part2 + (i - n1);
+            const int64_t step = i < n1 ? n1 : n2;
 #pragma unroll 8
-        for (int z = 0; z < slices; ++z)
-            acc += p[z * step];
-        G[1 + i] += acc;
+            for (int z = warp; z < slices; z += 8)
+                acc += p[z * step];
+        }
+        sums[warp][lane] = acc;
+        __syncthreads();
+        if (warp == 0 && i < n1 + n2) {
+#pragma unroll
+            for (int w = 1; w < 8; ++w)
+                acc += sums[w][lane];
+            G[1 + i] += acc;
+        }
+        __syncthreads();
     }
 }
 
@@ -687,11 +712,11 @@ cudaError_t launch_entry_labels(const uint32_t *ids, int k, int64_t n, const uin
     return cudaGetLastError();
 }
 
-// Samples of one gradient pass: as many as keep a chunk's working memory at about 32 MB
+// Samples of one gradient pass: as many as keep a chunk's working memory at about 64 MB
 // (it then stays in L2 between the kernels), in whole slices and at least 2,048.
 int entry_train_chunk(int64_t n, int d, int E) {
     const int64_t per = 2 * EH + E + ((int64_t)(d + 1) * EH + (int64_t)(EH + 1) * E) / SLICE + 1;
-    int64_t B = (int64_t(8) << 20) / per / SLICE * SLICE;
+    int64_t B = (int64_t(16) << 20) / per / SLICE * SLICE;
     B = B < 2048 ? 2048 : B > 65536 ? 65536 : B;
     return (int)(n < B ? n : B);
 }
@@ -733,7 +758,7 @@ cudaError_t entry_grad_accumulate(const float *P, int d, int E, const float *X,
         train_dz_kernel<<<bt, 256, 0, s>>>(P, H, T, nb, E, dZ, L);
         train_gw_kernel<<<dim3(1, (unsigned)((d + GT) / GT), sl), 256, 0, s>>>(Xb, d, P, dZ, EH,
                                                                               nb, part1);
-        grad_reduce_kernel<<<grid_for(n1 + n2, 256), 256, 0, s>>>(part1, n1, part2, n2, (int)sl,
+        grad_reduce_kernel<<<grid_for(n1 + n2, 32), 256, 0, s>>>(part1, n1, part2, n2, (int)sl,
                                                                   G);
         if ((e = cudaGetLastError()) != cudaSuccess)
             return e;
