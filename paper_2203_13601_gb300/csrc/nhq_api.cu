@@ -360,6 +360,84 @@ nhq_status nhq_pack_attributes(const uint8_t *attributes, int64_t n, int32_t m, 
     return NHQ_OK;
 }
 
+// the packed attribute words sorted ascending with their ids (stable), built once
+static nhq_status ensure_attribute_order(nhq_index *ix, cudaStream_t s) {
+    if (ix->attr_sorted != nullptr)
+        return NHQ_OK;
+    CKS(scratch(ix, attribute_sort_scratch_bytes(ix->N)));
+    uint32_t *words = nullptr, *ids = nullptr;
+    cudaError_t e = cudaMalloc(&words, sizeof(uint32_t) * (size_t)ix->N);
+    if (e == cudaSuccess)
+        e = cudaMalloc(&ids, sizeof(uint32_t) * (size_t)ix->N);
+    if (e == cudaSuccess)
+        e = launch_attribute_sort(ix->attr, ix->N, words, ids, ix->scratch, ix->scratch_bytes, s);
+    if (e != cudaSuccess) {
+        cudaFree(words);
+        cudaFree(ids);
+        return fail_cuda(e, "attribute order");
+    }
+    ix->attr_sorted = words;
+    ix->id_sorted = ids;
+    return NHQ_OK;
+}
+
+static bool is_capturing(cudaStream_t s) {
+    cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(s, &st) != cudaSuccess) {
+        cudaGetLastError();
+        return true;
+    }
+    return st != cudaStreamCaptureStatusNone;
+}
+
+// Whether an exact top-k over all objects takes the tuple runs of the attribute order.
+// They cost four to seven launches against the scan's three, so a scan of less than 2^26
+// pair dimensions (under 20 us) is left alone; where the order does not exist yet, sorting
+// the words and allocating it (about 0.3 ms once) has to pay in this very call.  Nothing is
+// allocated while a capture is running: what is there already decides.
+static bool take_runs(const nhq_index *ix, const TopkArgs &a, bool capturing) {
+    if (!topk_runs_apply(a))
+        return false;
+    const double work = (double)a.nq * (double)a.N * (double)a.d;
+    if (capturing)
+        return ix->attr_sorted != nullptr &&
+               topk_runs_scratch_bytes(a, ix->sm_count) <= ix->scratch_bytes &&
+               work >= (double)(1 << 26);
+    return work >= (ix->attr_sorted != nullptr ? (double)(1 << 26) : (double)(1 << 29));
+}
+
+// The exact top-k of a.nq queries in the index's scratch; codes: the queries' attribute
+// codes (their words are packed here), or null when a.qattr holds the words.
+static nhq_status exact_topk(nhq_index *ix, TopkArgs a, const uint8_t *codes, cudaStream_t s) {
+    const bool capturing = is_capturing(s);
+    if (take_runs(ix, a, capturing)) {
+        if (capturing || (ensure_attribute_order(ix, s) == NHQ_OK &&
+                          scratch(ix, topk_runs_scratch_bytes(a, ix->sm_count)) == NHQ_OK)) {
+            CK(launch_topk_runs(a, codes, ix->attr_sorted, ix->id_sorted, ix->scratch,
+                                ix->scratch_bytes, ix->sm_count, s));
+            return NHQ_OK;
+        }
+        cudaGetLastError();  // no memory for the order or the runs' lists: the scan answers
+    }
+    // query words, then (with a wildcard) their chi masks, then the slices' lists
+    const size_t row = ((sizeof(uint32_t) * (size_t)a.nq) + 255) & ~(size_t)255;
+    const size_t words = codes == nullptr ? 0 : a.w.wild ? 2 * row : row;
+    size_t need = words + topk_scratch_bytes(a, ix->sm_count);
+    if (capturing && need > ix->scratch_bytes)  // fewer slices in what there is
+        need = words > ix->scratch_bytes ? words : ix->scratch_bytes;
+    CKS(scratch(ix, need));
+    if (codes != nullptr) {
+        uint32_t *qa = reinterpret_cast<uint32_t *>(ix->scratch);
+        uint32_t *qh =
+            a.w.wild ? reinterpret_cast<uint32_t *>((char *)ix->scratch + row) : nullptr;
+        CK(launch_pack_queries(codes, a.nq, a.w, qa, qh, s));
+        a.qattr = qa;
+        a.qhi = qh;
+    }
+    CK(launch_topk(a, (char *)ix->scratch + words, ix->scratch_bytes - words, ix->sm_count, s));
+    return NHQ_OK;
+}
+
 nhq_status nhq_knn(const nhq_index *cix, int32_t K, uint32_t *cand_ids, float *cand_dist,
                    void *stream) {
     nhq_index *ix = const_cast<nhq_index *>(cix);
@@ -389,22 +467,8 @@ nhq_status nhq_knn(const nhq_index *cix, int32_t K, uint32_t *cand_ids, float *c
     a.ids = (uint32_t *)st.dev(io);
     a.dists = (float *)st.dev(id);
     a.chi = nullptr;
-    size_t need = topk_scratch_bytes(a, ix->sm_count);
-    CKS(scratch(ix, need + 256));
-    CK(launch_topk(a, ix->scratch, ix->scratch_bytes, ix->sm_count, s));
+    CKS(exact_topk(ix, a, nullptr, s));
     return st.finish(s);
-}
-
-// the packed attribute words sorted ascending with their ids (stable), built once
-static nhq_status ensure_attribute_order(nhq_index *ix, cudaStream_t s) {
-    if (ix->attr_sorted != nullptr)
-        return NHQ_OK;
-    CK(cudaMalloc(&ix->attr_sorted, sizeof(uint32_t) * (size_t)ix->N));
-    CK(cudaMalloc(&ix->id_sorted, sizeof(uint32_t) * (size_t)ix->N));
-    CKS(scratch(ix, attribute_sort_scratch_bytes(ix->N)));
-    CK(launch_attribute_sort(ix->attr, ix->N, ix->attr_sorted, ix->id_sorted, ix->scratch,
-                             ix->scratch_bytes, s));
-    return NHQ_OK;
 }
 
 nhq_status nhq_knn_bf16(const nhq_index *cix, int32_t K, uint32_t *cand_ids, float *cand_dist,
@@ -971,6 +1035,8 @@ nhq_status nhq_brute_force_wildcard(const nhq_index *cix, const float *queries,
     a.attr = ix->attr;
     a.Q = (const float *)st.dev(iq);
     a.qstride = ix->d;
+    a.qattr = nullptr;
+    a.qhi = nullptr;
     a.nq = Q;
     a.k = k;
     a.exclude_self = 0;
@@ -979,19 +1045,7 @@ nhq_status nhq_brute_force_wildcard(const nhq_index *cix, const float *queries,
     a.ids = (uint32_t *)st.dev(io);
     a.dists = (float *)st.dev(id);
     a.chi = (uint8_t *)st.dev(ic);
-    // query words, then (with a wildcard) their chi masks
-    size_t qa_bytes = ((sizeof(uint32_t) * (size_t)Q) + 255) & ~(size_t)255;
-    const size_t words = wildcard ? 2 * qa_bytes : qa_bytes;
-    size_t need = words + topk_scratch_bytes(a, ix->sm_count);
-    CKS(scratch(ix, need));
-    uint32_t *qa = reinterpret_cast<uint32_t *>(ix->scratch);
-    uint32_t *qh = wildcard ? reinterpret_cast<uint32_t *>((char *)ix->scratch + qa_bytes) : nullptr;
-    CK(launch_pack_queries((const uint8_t *)st.dev(ia), Q, a.w, qa, qh, s));
-    a.qattr = qa;
-    a.qhi = qh;
-    qa_bytes = words;
-    CK(launch_topk(a, (char *)ix->scratch + qa_bytes, ix->scratch_bytes - qa_bytes, ix->sm_count,
-                   s));
+    CKS(exact_topk(ix, a, (const uint8_t *)st.dev(ia), s));
     return st.finish(s);
 }
 

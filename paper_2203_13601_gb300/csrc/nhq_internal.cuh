@@ -243,6 +243,13 @@ struct TopkArgs {
 size_t topk_scratch_bytes(const TopkArgs &a, int sm_count);
 cudaError_t launch_topk(const TopkArgs &a, void *scratch, size_t scratch_bytes, int sm_count,
                         cudaStream_t s);
+// the same answer from the tuple runs of the attribute order (filter and constant weights,
+// closed queries); codes: the queries' attributes, or null when a.qattr holds their words
+bool topk_runs_apply(const TopkArgs &a);
+size_t topk_runs_scratch_bytes(const TopkArgs &a, int sm_count);
+cudaError_t launch_topk_runs(const TopkArgs &a, const uint8_t *codes,
+                             const uint32_t *attr_sorted, const uint32_t *id_sorted,
+                             void *scratch, size_t scratch_bytes, int sm_count, cudaStream_t s);
 
 // k_edge.cu
 // landing-zone selection for the vertices rows[b] (or row0 + b), candidate row b -> out row b
