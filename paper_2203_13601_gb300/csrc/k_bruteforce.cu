@@ -21,12 +21,12 @@
 // through the full scan afterwards, counted on the device.
 //
 // What bounds it: the full scan the FP32 pipe and the issue slots around it.  Candidate
-// sets of 60,000 objects (d = 96, K = 64, proportional weights) take 44.8 ms, half the FP32
+// sets of 60,000 objects (d = 96, K = 64, proportional weights) take 41.2 ms, half the FP32
 // rate of a difference and an fma per dimension; before (no staging ahead, every pair's
 // Gamma with its division, records inserted one by one) 55.5 ms.  2,003 queries, k = 100,
-// over 300,007 objects: 11.4 ms, before 16.4 ms.  The runs do a hundredth of the pairs: the
-// filter truth of 10,000 queries over a million objects (600 tuples) 1.81 ms, before 206 ms;
-// eight queries under constant weights 72 us, before 5,560 us.
+// over 300,007 objects: 10.6 ms, before 16.4 ms.  The runs do a hundredth of the pairs: the
+// filter truth of 10,000 queries over a million objects (600 tuples) 1.67 ms, before 206 ms;
+// eight queries under constant weights 62 us, before 5,560 us.
 #include <cmath>
 #include <cstdio>
 #include <mutex>
@@ -98,6 +98,20 @@ __device__ __forceinline__ float admitted_dist2(float g, const Fusion &w) {
     else if (w.mode == NHQ_W_CONSTANT && w.wv > 1e-30f)
         s = (g / w.wv) * 1.00001f;
     return s * s * 1.00001f + 1e-36f;
+}
+
+// Two differences in one instruction, each rounded as a single one is: six issue slots for
+// four dimensions of a pair instead of eight (candidate sets of 60,000 objects 44.8 ->
+// 41.2 ms, filter truth of 10,000 queries 1.79 -> 1.65 ms).  The sums stay one chain.
+__device__ __forceinline__ unsigned long long sub2(unsigned long long a, unsigned long long b) {
+    unsigned long long d;
+    asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+    return d;
+}
+__device__ __forceinline__ void add_squares(float &acc, unsigned long long t) {
+    const float lo = __uint_as_float((uint32_t)t), hi = __uint_as_float((uint32_t)(t >> 32));
+    acc = fmaf(lo, lo, acc);
+    acc = fmaf(hi, hi, acc);
 }
 
 __device__ __forceinline__ void cp16(uint32_t dst, const void *src, int bytes) {
@@ -262,24 +276,19 @@ __device__ __forceinline__ void scan_objects(const TopkArgs &a, Smem<T> &sm,
             // differences one dimension at a time, in dimension order
 #pragma unroll 2
             for (int c = 0; c < DC; c += 4) {
-                float4 q[T::QI];
+                ulonglong2 q[T::QI];
 #pragma unroll
                 for (int i = 0; i < T::QI; ++i)
-                    q[i] = *reinterpret_cast<const float4 *>(&sm.st[buf].Q[ty + T::TY * i][c]);
+                    q[i] = *reinterpret_cast<const ulonglong2 *>(
+                        &sm.st[buf].Q[ty + T::TY * i][c]);
 #pragma unroll
                 for (int j = 0; j < T::OJ; ++j) {
-                    const float4 b =
-                        *reinterpret_cast<const float4 *>(&sm.st[buf].X[tx + T::TX * j][c]);
+                    const ulonglong2 b = *reinterpret_cast<const ulonglong2 *>(
+                        &sm.st[buf].X[tx + T::TX * j][c]);
 #pragma unroll
                     for (int i = 0; i < T::QI; ++i) {
-                        float t = q[i].x - b.x;
-                        acc[i][j] = fmaf(t, t, acc[i][j]);
-                        t = q[i].y - b.y;
-                        acc[i][j] = fmaf(t, t, acc[i][j]);
-                        t = q[i].z - b.z;
-                        acc[i][j] = fmaf(t, t, acc[i][j]);
-                        t = q[i].w - b.w;
-                        acc[i][j] = fmaf(t, t, acc[i][j]);
+                        add_squares(acc[i][j], sub2(q[i].x, b.x));
+                        add_squares(acc[i][j], sub2(q[i].y, b.y));
                     }
                 }
             }
