@@ -294,7 +294,17 @@ __global__ void __launch_bounds__(NTHREADS, 1)
     const uint32_t sbytes = resA ? BOX_BYTES : 2 * BOX_BYTES;
     const uint32_t boff = resA ? 0u : BOX_BYTES;  // B box within a stage
     unsigned char *aregion = ring + 4 * BOX_BYTES;
-    const int t0 = (int)blockIdx.x;  // the diagonal tile comes first
+    // The diagonal tile comes first, or under constant weights the one before it where the
+    // first row's tuple run began there and leaves fewer than K others in the diagonal tile:
+    // a row that has not met K objects of its own tuple keeps every tile alive, and the
+    // rest of its run would come last of all; runs of more than K objects are now met
+    // within two tiles (a build of 1M objects of 600 tuples 129.7 -> 125.0 ms).
+    int t0 = (int)blockIdx.x;
+    if (MODE == NHQ_W_CONSTANT && t0 > 0) {
+        const uint32_t first = a.attr[row0];
+        if (a.attr[row0 - 1] == first && !(row0 + a.K < a.N && a.attr[row0 + a.K] == first))
+            --t0;
+    }
     auto tile_at = [&](int i) { return t0 + i < ntiles ? t0 + i : t0 + i - ntiles; };
     auto bar = [&](int i) { return smem_u32(bars + i); };
     const int FULL0 = 0, EMPTY0 = MAX_STAGES, TFULL0 = 2 * MAX_STAGES, TEMPTY0 = TFULL0 + NBUF,
@@ -374,12 +384,25 @@ __global__ void __launch_bounds__(NTHREADS, 1)
         uint32_t wbits = 0u;       // skip bits of the current word, published by lane 0
         uint32_t dead_tuple = 0u;  // a tuple whose tiles were found dead (stays dead)
         bool have_dead = false;
+        // The objects that carry one of the rows' tuples are the sorted positions of tiles
+        // tlo..thi.  Once every row's bound for chi = 1 is negative (so for every larger chi:
+        // it falls with chi) all other tiles are dead, and the sweep goes to the next tile of
+        // that range in one step (found when first needed).
+        // At 1M objects of 600 tuples a CTA keeps about 110 of 7,813 tiles, and deciding
+        // the others tuple by tuple, some 1,000 serial decisions, took longer than the kept
+        // ones: the build went from 125.0 to 85.5 ms, its candidates from 73 to 29 ms.
+        bool closed = false;
+        int tlo = 0, thi = -1;
         int i = 0;
         while (i < ntiles && ok) {
             if ((i >> 5) != gcur) {
-                cf = nf;
-                cl = nl;
-                ++gcur;
+                if ((i >> 5) == gcur + 1) {
+                    cf = nf;
+                    cl = nl;
+                } else {
+                    codes((i >> 5) * 32, cf, cl);
+                }
+                gcur = i >> 5;
                 codes((gcur + 1) * 32, nf, nl);
             }
             const int j = i & 31;
@@ -415,6 +438,60 @@ __global__ void __launch_bounds__(NTHREADS, 1)
                 }
             }
             int step = 1;
+            if (skip_on && !need) {
+                if (!closed) {
+                    bool open = false;
+#pragma unroll
+                    for (int k = 0; k < 4; ++k)
+                        open = open || (rv[k] && !(reinterpret_cast<const volatile float *>(
+                                                       limtab)[BM + lane + 32 * k] < 0.f));
+                    closed = !__any_sync(0xFFFFFFFFu, open);
+                    if (closed) {
+                        // lane 0: first position of the first row's word; lane 1: first
+                        // position after the last row's word
+                        const int64_t last = row0 + BM < a.N ? row0 + BM - 1 : a.N - 1;
+                        const uint32_t word = a.attr[lane == 0 ? row0 : last];
+                        int64_t lo = lane == 0 ? 0 : last, hi = lane == 0 ? row0 : a.N;
+                        while (lo < hi) {
+                            const int64_t mid = (lo + hi) >> 1;
+                            const uint32_t x = a.attr[mid];
+                            if (lane == 0 ? x < word : x <= word)
+                                lo = mid + 1;
+                            else
+                                hi = mid;
+                        }
+                        tlo = (int)(__shfl_sync(0xFFFFFFFFu, lo, 0) / BN);
+                        thi = (int)((__shfl_sync(0xFFFFFFFFu, lo, 1) - 1) / BN);
+                    }
+                }
+                const int t = tile_at(i);
+                if (closed && (t < tlo || t > thi)) {
+                    // the sweep is t0 .. ntiles - 1, 0 .. t0 - 1, with tlo <= t0 + 1
+                    int to = ntiles;
+                    if (t < tlo && i + (tlo - t) < ntiles)
+                        to = i + (tlo - t);
+                    else if (t > thi && tlo < t0)
+                        to = ntiles - t0 + tlo;
+                    const int w0 = i >> 5, w1 = to >> 5;
+                    const uint32_t end = (1u << (to & 31)) - 1u;  // bits of word w1
+                    wbits |= (w0 == w1 ? end : 0xFFFFFFFFu) & ~((1u << j) - 1u);
+                    if (lane == 0)
+                        skipbits[w0] = wbits;
+                    for (int w = w0 + 1 + lane; w < w1; w += 32)
+                        skipbits[w] = 0xFFFFFFFFu;
+                    if (w1 != w0) {
+                        wbits = end;
+                        if (lane == 0 && end != 0u)
+                            skipbits[w1] = end;
+                    }
+                    __threadfence_block();
+                    __syncwarp();
+                    if (lane == 0)
+                        *reinterpret_cast<volatile int *>(decided) = to;
+                    i = to;
+                    continue;
+                }
+            }
             if (!need) {
                 // the following tiles of this group with the same first and last word
                 // are rejected by the same bounds
