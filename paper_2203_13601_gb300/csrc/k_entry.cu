@@ -323,15 +323,17 @@ __global__ void entry_to_half_kernel(const float *__restrict__ p, __half *__rest
 // gradients (4 and 2 tiles of outputs) split the samples into slices of SLICE, each
 // writing its own partial sums, which grad_reduce_kernel adds in slice order (no atomics:
 // the gradient is the same in every run).  That step took 2,804 us with one thread per
-// output walking all samples of a 2,048-sample chunk in eight chunks, and takes 158 us.
+// output walking all samples of a 2,048-sample chunk in eight chunks, and takes 133 us.
 constexpr int GT = 64, GK = 32, GP = GT + 1;
 constexpr int SLICE = 128;
 
 // acc[i][j] (+)= sum over k in [k0, k1) of a(k, ty * 4 + i) b(k, tx * 4 + j), k ascending.
 // AK / BK: the operand is contiguous along k in memory (the staging loop follows it).
+// sum (or null): the threads with ty = 0 also add b(k, tx + 16 j) over k into sum[j].
 template <bool AK, bool BK, class LA, class LB>
 __device__ __forceinline__ void tile_product(float acc[4][4], int64_t k0, int64_t k1, LA la, LB lb,
-                                             float (*As)[GP], float (*Bs)[GP]) {
+                                             float (*As)[GP], float (*Bs)[GP],
+                                             float *sum = nullptr) {
     const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
     float ra[8], rb[8];
     auto fetch = [&](int64_t kb) {
@@ -368,6 +370,11 @@ __device__ __forceinline__ void tile_product(float acc[4][4], int64_t k0, int64_
 #pragma unroll
                 for (int j = 0; j < 4; ++j)
                     acc[i][j] = fmaf(a[i], b[j], acc[i][j]);
+            if (sum != nullptr && ty == 0) {
+#pragma unroll
+                for (int j = 0; j < 4; ++j)
+                    sum[j] += b[j];
+            }
         }
         __syncthreads();
     }
@@ -513,8 +520,9 @@ __global__ void __launch_bounds__(256) train_dz_kernel(const float *__restrict__
 
 // Partial sums of one weight gradient over a slice of samples: part[slice][r][c] =
 // sum_b A[b][r] D[b][c] for r < rows (times the input scale when scale is set) and row
-// r = rows the plain sums of D (the bias).  A has rows values per sample, D cols;
-// grid (ceil(cols/64), ceil((rows+1)/64), slices).
+// r = rows the plain sums of D (the bias), which the first row of tiles adds up on the
+// side (as a row of the product it took a tile row of its own).  A has rows values per
+// sample, D cols; grid (ceil(cols/64), ceil(rows/64), slices).
 __global__ void __launch_bounds__(256) train_gw_kernel(const float *__restrict__ A, int rows,
                                                        const float *__restrict__ scale,
                                                        const float *__restrict__ D, int cols,
@@ -525,25 +533,24 @@ __global__ void __launch_bounds__(256) train_gw_kernel(const float *__restrict__
     const int64_t b0 = (int64_t)blockIdx.z * SLICE;
     const int64_t b1 = b0 + SLICE < B ? b0 + SLICE : B;
     const float s = scale != nullptr ? *scale : 1.f;
-    float acc[4][4] = {};
+    float acc[4][4] = {}, sum[4] = {};
     tile_product<false, false>(
-        acc, b0, b1,
-        [&](int64_t k, int r) {
-            return r0 + r < rows ? s * A[k * rows + r0 + r] : r0 + r == rows ? 1.f : 0.f;
-        },
-        [&](int64_t k, int c) { return c0 + c < cols ? D[k * cols + c0 + c] : 0.f; }, As, Bs);
+        acc, b0, b1, [&](int64_t k, int r) { return r0 + r < rows ? s * A[k * rows + r0 + r] : 0.f; },
+        [&](int64_t k, int c) { return c0 + c < cols ? D[k * cols + c0 + c] : 0.f; }, As, Bs, sum);
     float *out = part + (int64_t)blockIdx.z * (rows + 1) * cols;
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
-        const int r = r0 + ty * 4 + i;
-        if (r > rows)
+    for (int j = 0; j < 4; ++j) {
+        const int c = c0 + tx + 16 * j;
+        if (c >= cols)
             continue;
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            const int c = c0 + tx + 16 * j;
-            if (c < cols)
+        for (int i = 0; i < 4; ++i) {
+            const int r = r0 + ty * 4 + i;
+            if (r < rows)
                 out[(int64_t)r * cols + c] = acc[i][j];
         }
+        if (ty == 0 && r0 == 0)
+            out[(int64_t)rows * cols + c] = sum[j];
     }
 }
 
@@ -753,10 +760,10 @@ cudaError_t entry_grad_accumulate(const float *P, int d, int E, const float *X,
         train_hidden_kernel<<<bt, 256, 0, s>>>(P, Xb, nb, d, H, L);
         train_out_kernel<<<dim3(bt, et), 256, 0, s>>>(P, H, nb, E, T, L);
         train_softmax_kernel<<<(nb + 7) / 8, 256, 0, s>>>(T, y + b0, nb, E, inv, loss);
-        train_gw_kernel<<<dim3(et, (EH + GT) / GT, sl), 256, 0, s>>>(H, EH, nullptr, T, E, nb,
+        train_gw_kernel<<<dim3(et, EH / GT, sl), 256, 0, s>>>(H, EH, nullptr, T, E, nb,
                                                                     part2);
         train_dz_kernel<<<bt, 256, 0, s>>>(P, H, T, nb, E, dZ, L);
-        train_gw_kernel<<<dim3(1, (unsigned)((d + GT) / GT), sl), 256, 0, s>>>(Xb, d, P, dZ, EH,
+        train_gw_kernel<<<dim3(1, (unsigned)((d + GT - 1) / GT), sl), 256, 0, s>>>(Xb, d, P, dZ, EH,
                                                                               nb, part1);
         grad_reduce_kernel<<<grid_for(n1 + n2, 32), 256, 0, s>>>(part1, n1, part2, n2, (int)sl,
                                                                   G);
