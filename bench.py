@@ -218,19 +218,19 @@ def fp32_simt_peak(dev):
 
 
 def brute_force_roofline(nhq, ix, Qv, QA, k, n, d, dev, stream):
-    """The brute-force fused top-k (every query against every object, constant weights)
-    timed with CUDA events on its stream: 3 flops per (query, object, dimension) (the
+    """The brute-force fused top-k (every query against every object: the default weighting,
+    under which no tuple is ruled out) timed with CUDA events on its stream: 3 flops per (query, object, dimension) (the
     difference and its fused square-add) against the measured SGEMM rate."""
     import torch
 
     nq = Qv.shape[0]
     ids = torch.empty((nq, k), dtype=torch.uint32, device=dev)
-    nhq.nhq_brute_force(ix.handle, Qv, QA, k, ids, weights=CONST_W, stream=stream)
+    nhq.nhq_brute_force(ix.handle, Qv, QA, k, ids, weights=None, stream=stream)
     e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
     reps = 2
     e0.record(stream)
     for _ in range(reps):
-        nhq.nhq_brute_force(ix.handle, Qv, QA, k, ids, weights=CONST_W, stream=stream)
+        nhq.nhq_brute_force(ix.handle, Qv, QA, k, ids, weights=None, stream=stream)
     e1.record(stream)
     e1.synchronize()
     ms = e0.elapsed_time(e1) / reps

@@ -390,7 +390,7 @@ __global__ void __launch_bounds__(NTHREADS, 1)
         // that range in one step (found when first needed).
         // At 1M objects of 600 tuples a CTA keeps about 110 of 7,813 tiles, and deciding
         // the others tuple by tuple, some 1,000 serial decisions, took longer than the kept
-        // ones: the build went from 125.0 to 85.5 ms, its candidates from 73 to 29 ms.
+        // ones: this kernel 73.4 -> 28.8 ms, the whole build 129.7 -> 85.5 ms.
         bool closed = false;
         int tlo = 0, thi = -1;
         int i = 0;
