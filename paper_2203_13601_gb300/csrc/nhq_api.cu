@@ -322,6 +322,7 @@ void nhq_free(nhq_index *ix) {
     cudaFree(ix->nbr_attr);
     cudaFree(ix->Xk);
     cudaFree(ix->normk);
+    cudaFree(ix->exact);
     cudaFree(ix->attr_sorted);
     cudaFree(ix->id_sorted);
     cudaFree(ix->cent);
@@ -361,16 +362,18 @@ nhq_status nhq_pack_attributes(const uint8_t *attributes, int64_t n, int32_t m, 
 }
 
 // the packed attribute words sorted ascending with their ids (stable), built once
-static nhq_status ensure_attribute_order(nhq_index *ix, cudaStream_t s) {
+// (sorted in the given arena)
+static nhq_status make_attribute_order(nhq_index *ix, void **arena, size_t *arena_bytes,
+                                       cudaStream_t s) {
     if (ix->attr_sorted != nullptr)
         return NHQ_OK;
-    CKS(scratch(ix, attribute_sort_scratch_bytes(ix->N)));
+    CKS(grow(arena, arena_bytes, attribute_sort_scratch_bytes(ix->N)));
     uint32_t *words = nullptr, *ids = nullptr;
     cudaError_t e = cudaMalloc(&words, sizeof(uint32_t) * (size_t)ix->N);
     if (e == cudaSuccess)
         e = cudaMalloc(&ids, sizeof(uint32_t) * (size_t)ix->N);
     if (e == cudaSuccess)
-        e = launch_attribute_sort(ix->attr, ix->N, words, ids, ix->scratch, ix->scratch_bytes, s);
+        e = launch_attribute_sort(ix->attr, ix->N, words, ids, *arena, *arena_bytes, s);
     if (e != cudaSuccess) {
         cudaFree(words);
         cudaFree(ids);
@@ -379,6 +382,10 @@ static nhq_status ensure_attribute_order(nhq_index *ix, cudaStream_t s) {
     ix->attr_sorted = words;
     ix->id_sorted = ids;
     return NHQ_OK;
+}
+
+static nhq_status ensure_attribute_order(nhq_index *ix, cudaStream_t s) {
+    return make_attribute_order(ix, &ix->scratch, &ix->scratch_bytes, s);
 }
 
 static bool is_capturing(cudaStream_t s) {
@@ -401,20 +408,22 @@ static bool take_runs(const nhq_index *ix, const TopkArgs &a, bool capturing) {
     const double work = (double)a.nq * (double)a.N * (double)a.d;
     if (capturing)
         return ix->attr_sorted != nullptr &&
-               topk_runs_scratch_bytes(a, ix->sm_count) <= ix->scratch_bytes &&
+               topk_runs_scratch_bytes(a, ix->sm_count) <= ix->exact_bytes &&
                work >= (double)(1 << 26);
     return work >= (ix->attr_sorted != nullptr ? (double)(1 << 26) : (double)(1 << 29));
 }
 
-// The exact top-k of a.nq queries in the index's scratch; codes: the queries' attribute
-// codes (their words are packed here), or null when a.qattr holds the words.
+// The exact top-k of a.nq queries, in working memory of its own; codes: the queries'
+// attribute codes (their words are packed here), or null when a.qattr holds the words.
 static nhq_status exact_topk(nhq_index *ix, TopkArgs a, const uint8_t *codes, cudaStream_t s) {
     const bool capturing = is_capturing(s);
     if (take_runs(ix, a, capturing)) {
-        if (capturing || (ensure_attribute_order(ix, s) == NHQ_OK &&
-                          scratch(ix, topk_runs_scratch_bytes(a, ix->sm_count)) == NHQ_OK)) {
-            CK(launch_topk_runs(a, codes, ix->attr_sorted, ix->id_sorted, ix->scratch,
-                                ix->scratch_bytes, ix->sm_count, s));
+        if (capturing ||
+            (make_attribute_order(ix, &ix->exact, &ix->exact_bytes, s) == NHQ_OK &&
+             grow(&ix->exact, &ix->exact_bytes, topk_runs_scratch_bytes(a, ix->sm_count)) ==
+                 NHQ_OK)) {
+            CK(launch_topk_runs(a, codes, ix->attr_sorted, ix->id_sorted, ix->exact,
+                                ix->exact_bytes, ix->sm_count, s));
             return NHQ_OK;
         }
         cudaGetLastError();  // no memory for the order or the runs' lists: the scan answers
@@ -423,18 +432,26 @@ static nhq_status exact_topk(nhq_index *ix, TopkArgs a, const uint8_t *codes, cu
     const size_t row = ((sizeof(uint32_t) * (size_t)a.nq) + 255) & ~(size_t)255;
     const size_t words = codes == nullptr ? 0 : a.w.wild ? 2 * row : row;
     size_t need = words + topk_scratch_bytes(a, ix->sm_count);
-    if (capturing && need > ix->scratch_bytes)  // fewer slices in what there is
-        need = words > ix->scratch_bytes ? words : ix->scratch_bytes;
-    CKS(scratch(ix, need));
+    void **arena = &ix->exact;
+    size_t *bytes = &ix->exact_bytes;
+    if (capturing && need > *bytes) {  // fewer slices, in what there is
+        if (ix->scratch_bytes > *bytes) {
+            arena = &ix->scratch;
+            bytes = &ix->scratch_bytes;
+        }
+        if (need > *bytes)
+            need = words > *bytes ? words : *bytes;
+    }
+    CKS(grow(arena, bytes, need));
+    char *base = reinterpret_cast<char *>(*arena);
     if (codes != nullptr) {
-        uint32_t *qa = reinterpret_cast<uint32_t *>(ix->scratch);
-        uint32_t *qh =
-            a.w.wild ? reinterpret_cast<uint32_t *>((char *)ix->scratch + row) : nullptr;
+        uint32_t *qa = reinterpret_cast<uint32_t *>(base);
+        uint32_t *qh = a.w.wild ? reinterpret_cast<uint32_t *>(base + row) : nullptr;
         CK(launch_pack_queries(codes, a.nq, a.w, qa, qh, s));
         a.qattr = qa;
         a.qhi = qh;
     }
-    CK(launch_topk(a, (char *)ix->scratch + words, ix->scratch_bytes - words, ix->sm_count, s));
+    CK(launch_topk(a, base == nullptr ? nullptr : base + words, *bytes - words, ix->sm_count, s));
     return NHQ_OK;
 }
 

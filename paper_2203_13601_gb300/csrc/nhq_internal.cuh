@@ -186,6 +186,10 @@ struct nhq_index {
     // scratch arena (grown on demand, owned by the index)
     void *scratch = nullptr;
     size_t scratch_bytes = 0;
+    // working memory of the exact top-k: apart from scratch, whose address a captured
+    // search keeps, so that an exact query between its launches does not move it
+    void *exact = nullptr;
+    size_t exact_bytes = 0;
 };
 
 namespace nhq {

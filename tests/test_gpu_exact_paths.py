@@ -122,3 +122,25 @@ def test_entry_gradient_at_the_edges_of_its_tiles(nhq, d, E, n):
     # f32 sums of at most 1,025 terms: relative 1e-4 of each sum's largest terms
     assert abs(loss.item() - lw * frac) <= 1e-4 * max(abs(lw), 1e-3)
     assert np.allclose(grad.cpu().numpy(), gw * frac, rtol=1e-3, atol=1e-5 * np.abs(gw).max())
+
+
+def test_exact_queries_leave_a_captured_search_alone(nhq):
+    # the exact calls' working memory is larger than the search's, whose address the
+    # captured search keeps
+    w = synth.int_valued(20000, 3000, 16, cards=(2, 3), n_comp=9, seed=8)
+    q = 50
+    with nhq.Index.build(dev(w.X), dev(w.A), degree=16, weights=CONST, K=32) as ix:
+        ids, g, chi = empty_out(q, 10)
+        Qv, QA = dev(w.Qv[:q]), dev(w.QA[:q])  # the captured search reads them at every launch
+        graph = nhq.nhq_search_graph_create(ix.handle, Qv, QA, 10, 32, ids, g, chi, seed=1,
+                                            seed_mode=nhq.SEED_ATTRIBUTE)
+        torch.cuda.synchronize()
+        want = ids_i64(ids), g.cpu().numpy().copy()
+        for weights in ("filter", "index", None):
+            _check(nhq, w, 10, weights, CONST if weights == "index" else weights, ix)
+        ids.zero_()
+        g.zero_()
+        graph.launch()
+        torch.cuda.synchronize()
+        assert (ids_i64(ids) == want[0]).all() and np.array_equal(g.cpu().numpy(), want[1])
+        graph.close()
