@@ -31,7 +31,7 @@
 #include <cstdio>
 #include <mutex>
 
-#include "nhq_internal.cuh"
+#include "topk_plan.cuh"
 
 namespace nhq {
 
@@ -519,7 +519,7 @@ __global__ void scan_merge_kernel(TopkArgs a, ScanQueries sq, int tq,
 // group then claims the group's place among the groups, units (query tile x slice of the
 // run), query slots and list rows in single additions.
 struct RunHeader {
-    unsigned long long groups_units;  // groups << 40 | units: group order is unit order
+    unsigned long long groups_units;  // see plan_claim
     unsigned long long list_rows;
     unsigned slots, left, next;
 };
@@ -545,7 +545,6 @@ struct RunPlan {
     uint32_t *words;
     int tq, slice;  // queries per unit, objects per slice aimed at
 };
-constexpr int kUnitBits = 40;
 
 __device__ __forceinline__ int64_t lower_bound_word(const uint32_t *a, int64_t n, uint32_t x) {
     int64_t lo = 0, hi = n;
@@ -603,10 +602,10 @@ __device__ __forceinline__ void plan_group(const RunPlan &p, int64_t q) {
     }
     g.slices = (int)s;
     const unsigned long long units = (unsigned long long)((g.cnt + p.tq - 1) / p.tq) * s;
-    const unsigned long long at = atomicAdd(&p.hdr->groups_units, (1ull << kUnitBits) + units);
-    g.ubase = at & ((1ull << kUnitBits) - 1);
+    const unsigned long long at = atomicAdd(&p.hdr->groups_units, plan_claim(units));
+    g.ubase = claimed_units(at);
     g.pad = 0;
-    const uint32_t gi = (uint32_t)(at >> kUnitBits);
+    const uint32_t gi = (uint32_t)claimed_groups(at);
     p.group[gi] = g;
     p.tgroup[p.home[q]] = gi;
 }
@@ -656,8 +655,8 @@ __global__ void __launch_bounds__(NT, T::CTAS) run_kernel(TopkArgs a, RunPlan p)
     unsigned long long *lists = reinterpret_cast<unsigned long long *>(smem + sizeof(Smem<T>));
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const unsigned long long gu = p.hdr->groups_units;
-    const int64_t groups = (int64_t)(gu >> kUnitBits);
-    const int64_t units = (int64_t)(gu & ((1ull << kUnitBits) - 1));
+    const int64_t groups = (int64_t)claimed_groups(gu);
+    const int64_t units = (int64_t)claimed_units(gu);
     for (;;) {
         __syncthreads();  // the previous unit's lists are written
         if (tid == 0)
