@@ -41,7 +41,6 @@ constexpr int TN = 128;     // objects per tile
 constexpr int DC = 32;      // dimensions per staged chunk
 constexpr int DS = DC + 4;  // staged row stride: 16-byte aligned rows, read as float4
 constexpr int NT = 256;     // threads per CTA
-constexpr int MAX_SLICES = 128;
 constexpr unsigned FULL = 0xFFFFFFFFu;
 constexpr float INF = __builtin_huge_valf();
 constexpr unsigned long long NO_RECORD = (0x7F800000ull << 32) | kNone;  // (inf, none)
@@ -592,13 +591,11 @@ __device__ __forceinline__ void plan_group(const RunPlan &p, int64_t q) {
     g.len = p.len[q];
     g.cnt = p.tcnt[p.home[q]];
     g.base = atomicAdd(&p.hdr->slots, g.cnt);
-    int64_t s = ((int64_t)g.len + p.slice - 1) / p.slice;
-    s = s > MAX_SLICES ? MAX_SLICES : s;
+    int64_t s = run_slices(g.len, p.slice);
     g.lbase = 0;
-    if (s > 1) {  // a group whose lists do not fit takes its run in one slice
+    if (s > 1) {
         g.lbase = atomicAdd(&p.hdr->list_rows, (unsigned long long)g.cnt * s);
-        if (g.lbase + g.cnt * s > (unsigned long long)p.rows)
-            s = 1;
+        s = slices_with_room(s, g.cnt, g.lbase, p.rows);
     }
     g.slices = (int)s;
     const unsigned long long units = (unsigned long long)((g.cnt + p.tq - 1) / p.tq) * s;
@@ -803,12 +800,11 @@ ScanPlan plan_scan(int64_t nq, int k, int sm_count) {
     return p;
 }
 
-// List rows of a scan of nq queries, or (counted) of at most nq: t tiles take slices only
-// while t < ctas, and then make at most ctas units.
+// List rows of a scan of nq queries, or (counted) of at most nq: t tiles that take slices
+// make at most ctas units of a tile's rows.
 int64_t scan_rows(const ScanPlan &p, int64_t nq, int64_t N, bool counted) {
-    const int64_t tiles = (nq + p.shape - 1) / p.shape;
     if (counted)
-        return (p.sq.ctas + (tiles < p.sq.ctas ? tiles : p.sq.ctas)) * p.shape;
+        return (int64_t)p.sq.ctas * p.shape;
     const int S = scan_slices(nq, p.shape, N, p.sq.ctas, p.sq.max_s);
     return S > 1 ? nq * S : 0;
 }
@@ -857,17 +853,13 @@ struct RunLayout {
     int64_t rows, srows;
 };
 
-// List rows of the runs: 64 units of 32 queries for each SM, and two slices of every query
-// up to a million rows; a group that finds no room scans its run in one slice.
 RunLayout run_layout(const TopkArgs &a, int sm_count) {
     RunLayout L;
     uint64_t T = 64;
     while (T < 2 * (uint64_t)a.nq)
         T <<= 1;
     L.tmask = (uint32_t)(T - 1);
-    L.rows = (a.nq < (1 << 19) ? 2 * a.nq : 1 << 20) + 64 * (int64_t)sm_count * 32;
-    const int64_t all = a.nq * MAX_SLICES;
-    L.rows = L.rows < all ? L.rows : all;
+    L.rows = run_list_rows(a.nq, a.N, a.k, sm_count);
     L.srows = a.w.mode == NHQ_W_FILTER
                   ? 0
                   : scan_rows(plan_scan(a.nq, a.k, sm_count), a.nq, a.N, true);
@@ -947,12 +939,10 @@ cudaError_t launch_topk_runs(const TopkArgs &args, const uint8_t *codes,
     p.codes = codes;
     if (codes != nullptr)
         a.qattr = p.words;
-    // Few queries hardly share tuples: tiles of 4, and short slices so that one query's run
-    // fills the chip (9,000 objects on average at a million and 600 tuples: 36 slices of
-    // 256).  Larger batches fill it with tiles of 32 queries and pay for slices in lists.
+    // Few queries hardly share tuples: tiles of 4.
     const bool few = a.nq <= 64;
     p.tq = few ? Narrow::TQ : Mid::TQ;
-    p.slice = few ? 256 : a.nq <= 2048 ? 1024 : 2048;
+    p.slice = run_slice_length(a.nq);
     cudaError_t e;
     if (a.nq <= 2048) {
         run_plan_kernel<<<1, a.nq <= 256 ? 256 : 1024, 0, s>>>(a, p);

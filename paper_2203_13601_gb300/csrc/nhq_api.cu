@@ -639,8 +639,14 @@ nhq_status nhq_index_build(nhq_index *ix, int32_t degree, const nhq_build_params
     cudaStream_t s = as_stream(stream);
     uint32_t *cand = nullptr, *nbr = nullptr, *rc = nullptr;
     const size_t N = (size_t)ix->N;
+    const size_t exact_before = ix->exact_bytes;
     auto cleanup = [&]() {
         cudaStreamSynchronize(s);
+        if (ix->exact_bytes > exact_before) {  // f32 candidates: a serving index needs none
+            cudaFree(ix->exact);
+            ix->exact = nullptr;
+            ix->exact_bytes = 0;
+        }
         cudaFree(cand);
         cudaFree(nbr);
         cudaFree(rc);

@@ -22,4 +22,47 @@ __host__ __device__ inline uint64_t claimed_units(unsigned long long at) {
     return at & ((1ull << kUnitBits) - 1);
 }
 
+constexpr int MAX_SLICES = 128;
+
+// Objects per slice of a tuple's run.  Few queries hardly share tuples: short slices, so
+// that one query's run fills the chip (9,000 objects on average at a million and 600
+// tuples: 36 slices of 256).  Larger batches fill it with tiles of 32 queries and pay for
+// slices in lists.
+__host__ __device__ inline int run_slice_length(int64_t nq) {
+    return nq <= 64 ? 256 : nq <= 2048 ? 1024 : 2048;
+}
+
+__host__ __device__ inline int64_t run_slices(int64_t len, int slice) {
+    const int64_t s = (len + slice - 1) / slice;
+    return s > MAX_SLICES ? MAX_SLICES : s;
+}
+
+// Rows of k records kept for the lists of sliced runs: none where no run can take two
+// slices, never more than nq queries on the longest run could use, six for each query
+// (10,000 queries over a million objects of 600 tuples use five) or twelve tiles for each
+// SM, and at most 128 MB, since the index keeps them: 10,000 queries take 48 MB at k = 100
+// and 123 MB at k = 256.  (While neither N nor the bytes counted: 266 and 680 MB, and 658 MB
+// for 5,000 at k = 256 over 1,300 objects, which use none.  64 MB would cost the 10,000 at
+// k = 256 half their speed: 8.2 ms instead of 4.2.)
+constexpr size_t kRunListBytes = size_t(128) << 20;
+inline int64_t run_list_rows(int64_t nq, int64_t N, int k, int sm_count) {
+    const int64_t most = run_slices(N, run_slice_length(nq));
+    if (most == 1)
+        return 0;
+    const int64_t fill = 12 * (int64_t)sm_count * 32;
+    int64_t rows = 6 * nq > fill ? 6 * nq : fill;
+    rows = rows < nq * most ? rows : nq * most;
+    const int64_t fit = (int64_t)(kRunListBytes / ((sizeof(uint32_t) + sizeof(float)) * k));
+    return rows < fit ? rows : fit;
+}
+
+// Slices of a run that wants `want` of them for cnt queries and claimed cnt * want list
+// rows from `base` on, when there are `rows`: as many as fit; one slice needs no row.
+__host__ __device__ inline int64_t slices_with_room(int64_t want, int64_t cnt, uint64_t base,
+                                                    int64_t rows) {
+    const int64_t fit = base < (uint64_t)rows ? (rows - (int64_t)base) / cnt : 0;
+    const int64_t s = want < fit ? want : fit;
+    return s > 1 ? s : 1;
+}
+
 }  // namespace nhq

@@ -27,10 +27,35 @@ static int check_claims() {
     return 0;
 }
 
+// the rows kept for sliced runs: bounded in bytes and by what the runs can use, and never
+// handed out twice
+static int check_rows() {
+    for (int64_t nq : {1, 8, 64, 65, 2048, 2049, 5000, 10000, 1000000, 1 << 29})
+        for (int64_t N : {1, 256, 257, 1024, 1025, 1300, 2048, 2049, 70000, 1000000, 0x7FFFFFFE})
+            for (int k : {1, 10, 64, 100, 256}) {
+                const int64_t rows = run_list_rows(nq, N, k, 152);
+                const int64_t most = run_slices(N, run_slice_length(nq));
+                bool ok = rows >= 0 && rows <= nq * most && rows * 8 * k <= (128 << 20);
+                ok = ok && (most > 1 || rows == 0);
+                uint64_t base = 0;  // groups of ever more queries on the longest run
+                for (int64_t cnt = 1; cnt <= nq && ok; cnt = cnt * 3 + 1) {
+                    const int64_t s = slices_with_room(most, cnt, base, rows);
+                    ok = s >= 1 && s <= most && (s == 1 || (int64_t)base + s * cnt <= rows);
+                    base += (uint64_t)(cnt * most);
+                }
+                if (!ok)
+                    return std::printf("FAIL nq=%lld N=%lld k=%d rows=%lld\n", (long long)nq,
+                                       (long long)N, k, (long long)rows), 1;
+            }
+    return 0;
+}
+
 int main(int argc, char **argv) {
     int bad = 2;
     if (argc > 1 && !std::strcmp(argv[1], "claims"))
         bad = check_claims();
+    else if (argc > 1 && !std::strcmp(argv[1], "rows"))
+        bad = check_rows();
     if (bad == 0)
         std::printf("ok\n");
     return bad;

@@ -42,3 +42,77 @@ def test_more_than_2_24_tuples_in_one_batch(nhq):
         torch.cuda.synchronize()
     assert torch.equal(ids.view(torch.int32)[:, 0].long(), pick)
     assert not dist.any() and not chi.any()
+
+
+def _check(w, k, ids, g, weights, rows):
+    """Rows `rows` of a batch against the oracle, bit for bit (integer components)."""
+    got, gam = ids_i64(ids)[rows], g.cpu().numpy()[rows].astype(np.float64)
+    if weights == "filter":
+        want, wg, _ = O.filtered_topk(w.X, w.A, w.Qv[rows], w.QA[rows], k, prec=O.F32)
+    else:
+        want, wg, _ = O.fused_topk(w.X, w.A, w.Qv[rows], w.QA[rows], k, weights=weights,
+                                   prec=O.F32)
+    assert (got == want).all()
+    assert np.array_equal(gam[want >= 0], wg[want >= 0])
+
+
+@pytest.fixture(scope="module")
+def warm(nhq):
+    """The kernels are loaded (which takes device memory of its own)."""
+    w = synth.int_valued(9000, 3000, 32, cards=(2, 3), n_comp=9, seed=1)
+    X, A = dev(w.X), dev(w.A)
+    with nhq.Index.build(X, A, degree=16, weights=CONST, K=64) as ix:
+        for q in (700, 3000):
+            for weights in ("filter", "index"):
+                ids, g, chi = empty_out(q, 8)
+                nhq.nhq_brute_force(ix.handle, dev(w.Qv[:q]), dev(w.QA[:q]), 8, ids, g, chi,
+                                    weights=weights)
+    torch.cuda.synchronize()
+
+
+def _free():
+    torch.cuda.synchronize()
+    return torch.cuda.mem_get_info()[0]
+
+
+# rows of the lists: none (no run reaches two slices), then 48 and 123 MB, beside the plan's
+# tables of about 1 MB and, under constant weights, the lists of the queries that are left
+# for the scan (at most 20 MB); allocations come in 2 MB pages
+@pytest.mark.parametrize("N,nq,k,weights,limit", [
+    (1300, 5000, 256, "filter", 8), (60000, 10000, 100, "filter", 56),
+    (60000, 10000, 100, CONST, 80), (60000, 10000, 256, CONST, 152)])
+def test_working_memory_of_an_exact_batch(nhq, warm, N, nq, k, weights, limit):
+    w = synth.int_valued(N, nq, 32, cards=(2, 3), n_comp=9, seed=N)
+    with nhq.Index.create(dev(w.X), dev(w.A), CONST) as ix:
+        Qv, QA = dev(w.Qv), dev(w.QA)
+        ids, g, chi = empty_out(nq, k)
+        before = _free()
+        nhq.nhq_brute_force(ix.handle, Qv, QA, k, ids, g, chi,
+                            weights="filter" if weights == "filter" else "index")
+        assert before - _free() <= limit << 20
+        _check(w, k, ids, g, weights, np.arange(0, nq, 397))
+
+
+def test_runs_short_of_list_rows_take_fewer_slices(nhq):
+    # k = 256: 58,368 rows; one tuple asks for 4,000 x 44, small ones beside it
+    rng = np.random.default_rng(4)
+    w = synth.int_valued(100000, 4400, 12, cards=(2, 3, 4), n_comp=9, seed=9)
+    often = rng.random(w.N) < 0.9
+    w.A, w.QA = w.A.copy(), w.QA.copy()
+    w.A[often] = (1, 1, 1)
+    w.QA[:4000] = (1, 1, 1)
+    for weights in ("filter", CONST):
+        with nhq.Index.create(dev(w.X), dev(w.A), CONST) as ix:
+            ids, g, chi = empty_out(w.nq, 256)
+            nhq.nhq_brute_force(ix.handle, dev(w.Qv), dev(w.QA), 256, ids, g, chi,
+                                weights="filter" if weights == "filter" else "index")
+            _check(w, 256, ids, g, weights, np.r_[0:4000:211, 4000:4400:31])
+
+
+def test_an_f32_build_leaves_no_working_memory(nhq, warm):
+    w = synth.int_valued(30000, 8, 24, cards=(2, 3), n_comp=9, seed=3)
+    X, A = dev(w.X), dev(w.A)
+    before = _free()
+    with nhq.Index.build(X, A, degree=16, weights=CONST, K=64):
+        # rows of 32 floats, two adjacency arrays of 16, the attribute order, reverse lists
+        assert before - _free() <= 32 << 20
