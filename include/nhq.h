@@ -376,6 +376,8 @@ nhq_status nhq_build(const float *vectors, int64_t N, int32_t d, const uint8_t *
  * delta).  queries[Q][d] f32, query_attributes[Q][m] u8.  `w` overrides the
  * index weights when not NULL (NHQ_W_FILTER gives the hybrid ground truth of
  * Sec. 6.1).  ids[Q][k] u32, dists[Q][k] f32, chi[Q][k] u8 (may be NULL).
+ * With device pointers the call may be captured in a CUDA graph; the working memory
+ * that a captured call uses stays with the index until nhq_free.
  * Errors: k outside 1..256.
  */
 /* nhq_brute_force with the wildcard rule of nhq_search_params::wildcard (0 or 1). */

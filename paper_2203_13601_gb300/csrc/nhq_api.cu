@@ -5,6 +5,7 @@
 #include <cstdarg>
 #include <cstdio>
 #include <cstring>
+#include <new>
 #include <string>
 #include <vector>
 
@@ -323,6 +324,12 @@ void nhq_free(nhq_index *ix) {
     cudaFree(ix->Xk);
     cudaFree(ix->normk);
     cudaFree(ix->exact);
+    while (ix->exact_kept != nullptr) {
+        nhq_index::KeptBlock *b = ix->exact_kept;
+        ix->exact_kept = b->next;
+        cudaFree(b->block);
+        delete b;
+    }
     cudaFree(ix->attr_sorted);
     cudaFree(ix->id_sorted);
     cudaFree(ix->cent);
@@ -361,19 +368,16 @@ nhq_status nhq_pack_attributes(const uint8_t *attributes, int64_t n, int32_t m, 
     return NHQ_OK;
 }
 
-// the packed attribute words sorted ascending with their ids (stable), built once
-// (sorted in the given arena)
-static nhq_status make_attribute_order(nhq_index *ix, void **arena, size_t *arena_bytes,
+// the packed attribute words sorted ascending with their ids (stable), built once, in
+// `work` (attribute_sort_scratch_bytes)
+static nhq_status make_attribute_order(nhq_index *ix, void *work, size_t work_bytes,
                                        cudaStream_t s) {
-    if (ix->attr_sorted != nullptr)
-        return NHQ_OK;
-    CKS(grow(arena, arena_bytes, attribute_sort_scratch_bytes(ix->N)));
     uint32_t *words = nullptr, *ids = nullptr;
     cudaError_t e = cudaMalloc(&words, sizeof(uint32_t) * (size_t)ix->N);
     if (e == cudaSuccess)
         e = cudaMalloc(&ids, sizeof(uint32_t) * (size_t)ix->N);
     if (e == cudaSuccess)
-        e = launch_attribute_sort(ix->attr, ix->N, words, ids, *arena, *arena_bytes, s);
+        e = launch_attribute_sort(ix->attr, ix->N, words, ids, work, work_bytes, s);
     if (e != cudaSuccess) {
         cudaFree(words);
         cudaFree(ids);
@@ -385,7 +389,10 @@ static nhq_status make_attribute_order(nhq_index *ix, void **arena, size_t *aren
 }
 
 static nhq_status ensure_attribute_order(nhq_index *ix, cudaStream_t s) {
-    return make_attribute_order(ix, &ix->scratch, &ix->scratch_bytes, s);
+    if (ix->attr_sorted != nullptr)
+        return NHQ_OK;
+    CKS(scratch(ix, attribute_sort_scratch_bytes(ix->N)));
+    return make_attribute_order(ix, ix->scratch, ix->scratch_bytes, s);
 }
 
 static bool is_capturing(cudaStream_t s) {
@@ -397,20 +404,45 @@ static bool is_capturing(cudaStream_t s) {
     return st != cudaStreamCaptureStatusNone;
 }
 
+// Working memory of at least `need` bytes in ix->exact.  A captured call reads and writes
+// that block at every later launch, so from then on it is only ever put aside (see
+// nhq_index); a block is allocated in a running capture too, which the relaxed capture mode
+// of this thread allows.
+static nhq_status exact_room(nhq_index *ix, size_t need, bool capturing) {
+    if (ix->exact_bytes < need) {
+        if (ix->exact != nullptr && (capturing || ix->exact_captured)) {
+            auto *b = new (std::nothrow) nhq_index::KeptBlock{ix->exact, ix->exact_kept};
+            if (b == nullptr)
+                return fail(NHQ_ERR_OOM, "no memory for the exact query");
+            ix->exact_kept = b;
+            ix->exact = nullptr;
+            ix->exact_bytes = 0;
+            ix->exact_captured = false;
+        }
+        cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+        if (capturing)
+            CK(cudaThreadExchangeStreamCaptureMode(&mode));
+        const nhq_status st = grow(&ix->exact, &ix->exact_bytes, need);
+        if (capturing)
+            CK(cudaThreadExchangeStreamCaptureMode(&mode));
+        CKS(st);
+    }
+    ix->exact_captured = ix->exact_captured || capturing;
+    return NHQ_OK;
+}
+
 // Whether an exact top-k over all objects takes the tuple runs of the attribute order.
 // They cost four to seven launches against the scan's three, so a scan of less than 2^26
 // pair dimensions (under 20 us) is left alone; where the order does not exist yet, sorting
-// the words and allocating it (about 0.3 ms once) has to pay in this very call.  Nothing is
-// allocated while a capture is running: what is there already decides.
+// the words and allocating it (about 0.3 ms once) has to pay in this very call.  A capture
+// takes the order that is there: one made in it would be sorted at its launches only.
 static bool take_runs(const nhq_index *ix, const TopkArgs &a, bool capturing) {
     if (!topk_runs_apply(a))
         return false;
     const double work = (double)a.nq * (double)a.N * (double)a.d;
-    if (capturing)
-        return ix->attr_sorted != nullptr &&
-               topk_runs_scratch_bytes(a, ix->sm_count) <= ix->exact_bytes &&
-               work >= (double)(1 << 26);
-    return work >= (ix->attr_sorted != nullptr ? (double)(1 << 26) : (double)(1 << 29));
+    if (ix->attr_sorted != nullptr)
+        return work >= (double)(1 << 26);
+    return !capturing && work >= (double)(1 << 29);
 }
 
 // The exact top-k of a.nq queries, in working memory of its own; codes: the queries'
@@ -418,10 +450,10 @@ static bool take_runs(const nhq_index *ix, const TopkArgs &a, bool capturing) {
 static nhq_status exact_topk(nhq_index *ix, TopkArgs a, const uint8_t *codes, cudaStream_t s) {
     const bool capturing = is_capturing(s);
     if (take_runs(ix, a, capturing)) {
-        if (capturing ||
-            (make_attribute_order(ix, &ix->exact, &ix->exact_bytes, s) == NHQ_OK &&
-             grow(&ix->exact, &ix->exact_bytes, topk_runs_scratch_bytes(a, ix->sm_count)) ==
-                 NHQ_OK)) {
+        const size_t sort = ix->attr_sorted == nullptr ? attribute_sort_scratch_bytes(ix->N) : 0;
+        const size_t runs = topk_runs_scratch_bytes(a, ix->sm_count);
+        if (exact_room(ix, runs > sort ? runs : sort, capturing) == NHQ_OK &&
+            (sort == 0 || make_attribute_order(ix, ix->exact, ix->exact_bytes, s) == NHQ_OK)) {
             CK(launch_topk_runs(a, codes, ix->attr_sorted, ix->id_sorted, ix->exact,
                                 ix->exact_bytes, ix->sm_count, s));
             return NHQ_OK;
@@ -431,19 +463,10 @@ static nhq_status exact_topk(nhq_index *ix, TopkArgs a, const uint8_t *codes, cu
     // query words, then (with a wildcard) their chi masks, then the slices' lists
     const size_t row = ((sizeof(uint32_t) * (size_t)a.nq) + 255) & ~(size_t)255;
     const size_t words = codes == nullptr ? 0 : a.w.wild ? 2 * row : row;
-    size_t need = words + topk_scratch_bytes(a, ix->sm_count);
-    void **arena = &ix->exact;
-    size_t *bytes = &ix->exact_bytes;
-    if (capturing && need > *bytes) {  // fewer slices, in what there is
-        if (ix->scratch_bytes > *bytes) {
-            arena = &ix->scratch;
-            bytes = &ix->scratch_bytes;
-        }
-        if (need > *bytes)
-            need = words > *bytes ? words : *bytes;
-    }
-    CKS(grow(arena, bytes, need));
-    char *base = reinterpret_cast<char *>(*arena);
+    const size_t need = words + topk_scratch_bytes(a, ix->sm_count);
+    if (need > 0)
+        CKS(exact_room(ix, need, capturing));
+    char *base = reinterpret_cast<char *>(ix->exact);
     if (codes != nullptr) {
         uint32_t *qa = reinterpret_cast<uint32_t *>(base);
         uint32_t *qh = a.w.wild ? reinterpret_cast<uint32_t *>(base + row) : nullptr;
@@ -451,7 +474,8 @@ static nhq_status exact_topk(nhq_index *ix, TopkArgs a, const uint8_t *codes, cu
         a.qattr = qa;
         a.qhi = qh;
     }
-    CK(launch_topk(a, base == nullptr ? nullptr : base + words, *bytes - words, ix->sm_count, s));
+    CK(launch_topk(a, base == nullptr ? nullptr : base + words, ix->exact_bytes - words,
+                   ix->sm_count, s));
     return NHQ_OK;
 }
 

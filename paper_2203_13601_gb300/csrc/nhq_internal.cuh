@@ -187,9 +187,16 @@ struct nhq_index {
     void *scratch = nullptr;
     size_t scratch_bytes = 0;
     // working memory of the exact top-k: apart from scratch, whose address a captured
-    // search keeps, so that an exact query between its launches does not move it
+    // search keeps, so that an exact query between its launches does not move it.  A
+    // captured exact query keeps this address in turn: a block that a capture has used
+    // (exact_captured) is put aside when a larger one is needed, and freed with the index.
     void *exact = nullptr;
     size_t exact_bytes = 0;
+    bool exact_captured = false;
+    struct KeptBlock {
+        void *block;
+        KeptBlock *next;
+    } *exact_kept = nullptr;
 };
 
 namespace nhq {

@@ -1,4 +1,6 @@
 """The exact top-k where its plan and its working memory are at their limits."""
+import dataclasses
+
 import numpy as np
 import pytest
 
@@ -116,3 +118,41 @@ def test_an_f32_build_leaves_no_working_memory(nhq, warm):
     with nhq.Index.build(X, A, degree=16, weights=CONST, K=64):
         # rows of 32 floats, two adjacency arrays of 16, the attribute order, reverse lists
         assert before - _free() <= 32 << 20
+
+
+# the scan and the runs, captured before the index has working memory for them and after,
+# then replayed on new queries once larger eager calls have come between
+@pytest.mark.parametrize("weights,order", [(None, False), ("filter", True), (CONST, True),
+                                           (CONST, False)])
+@pytest.mark.parametrize("first", [False, True])
+def test_captured_exact_calls_outlive_larger_ones(nhq, warm, weights, order, first):
+    w = synth.int_valued(20000, 3000, 48, cards=(2, 3), n_comp=9, seed=13)
+    q = 600
+    how = "filter" if weights == "filter" else "index"
+    with nhq.Index.create(dev(w.X), dev(w.A), weights if weights == CONST else None) as ix:
+        if order:
+            nhq.nhq_index_build_cells(ix.handle, 4)
+        Qv, QA = dev(w.Qv[:q]), dev(w.QA[:q])
+        ids, g, chi = empty_out(q, 10)
+        if first:
+            nhq.nhq_brute_force(ix.handle, Qv[:40], QA[:40], 10, ids[:40], g[:40], chi[:40],
+                                weights=how)
+        torch.cuda.synchronize()
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph):
+            nhq.nhq_brute_force(ix.handle, Qv, QA, 10, ids, g, chi, weights=how)
+        big = empty_out(w.nq, 100)
+        for other in ("filter", "index"):
+            nhq.nhq_brute_force(ix.handle, dev(w.Qv), dev(w.QA), 100, *big, weights=other)
+            _check(w, 100, big[0], big[1], "filter" if other == "filter" else
+                   (CONST if weights == CONST else None), np.arange(0, w.nq, 501))
+        Qv.copy_(dev(w.Qv[q:2 * q]))
+        QA.copy_(dev(w.QA[q:2 * q]))
+        for _ in range(2):
+            ids.zero_()
+            g.zero_()
+            graph.replay()
+            torch.cuda.synchronize()
+            part = dataclasses.replace(w, Qv=w.Qv[q:2 * q], QA=w.QA[q:2 * q])
+            _check(part, 10, ids, g, weights, np.arange(0, q, 7))
+        del graph
