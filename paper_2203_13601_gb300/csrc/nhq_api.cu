@@ -368,8 +368,19 @@ nhq_status nhq_pack_attributes(const uint8_t *attributes, int64_t n, int32_t m, 
     return NHQ_OK;
 }
 
+static bool is_capturing(cudaStream_t s) {
+    cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(s, &st) != cudaSuccess) {
+        cudaGetLastError();
+        return true;
+    }
+    return st != cudaStreamCaptureStatusNone;
+}
+
 // the packed attribute words sorted ascending with their ids (stable), built once, in
-// `work` (attribute_sort_scratch_bytes)
+// `work` (attribute_sort_scratch_bytes).  Waits for the sort, as every later call takes the
+// order for ready, on whatever stream: an exact call on one stream may make it and a search
+// on another read seeds from it.
 static nhq_status make_attribute_order(nhq_index *ix, void *work, size_t work_bytes,
                                        cudaStream_t s) {
     uint32_t *words = nullptr, *ids = nullptr;
@@ -378,6 +389,8 @@ static nhq_status make_attribute_order(nhq_index *ix, void *work, size_t work_by
         e = cudaMalloc(&ids, sizeof(uint32_t) * (size_t)ix->N);
     if (e == cudaSuccess)
         e = launch_attribute_sort(ix->attr, ix->N, words, ids, work, work_bytes, s);
+    if (e == cudaSuccess && !is_capturing(s))
+        e = cudaStreamSynchronize(s);
     if (e != cudaSuccess) {
         cudaFree(words);
         cudaFree(ids);
@@ -393,15 +406,6 @@ static nhq_status ensure_attribute_order(nhq_index *ix, cudaStream_t s) {
         return NHQ_OK;
     CKS(scratch(ix, attribute_sort_scratch_bytes(ix->N)));
     return make_attribute_order(ix, ix->scratch, ix->scratch_bytes, s);
-}
-
-static bool is_capturing(cudaStream_t s) {
-    cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
-    if (cudaStreamIsCapturing(s, &st) != cudaSuccess) {
-        cudaGetLastError();
-        return true;
-    }
-    return st != cudaStreamCaptureStatusNone;
 }
 
 // Working memory of at least `need` bytes in ix->exact.  A captured call reads and writes

@@ -156,3 +156,29 @@ def test_captured_exact_calls_outlive_larger_ones(nhq, warm, weights, order, fir
             part = dataclasses.replace(w, Qv=w.Qv[q:2 * q], QA=w.QA[q:2 * q])
             _check(part, 10, ids, g, weights, np.arange(0, q, 7))
         del graph
+
+
+def test_attribute_order_of_an_exact_call_serves_other_streams(nhq):
+    # the candidate sets make the order on one stream; the search on the other one, which
+    # waits for nothing, takes its seeds from it
+    w = synth.int_valued(60000, 500, 32, cards=(3, 5), n_comp=9, seed=21)
+    X, A, Qv, QA = dev(w.X), dev(w.A), dev(w.Qv), dev(w.QA)
+    outs = []
+    with nhq.Index.build(X, A, degree=16, weights=CONST, K=32, knn_dtype=1) as built:
+        nbr = torch.empty((w.N, 16), dtype=torch.uint32, device="cuda:0")
+        nhq.nhq_index_get_graph(built.handle, nbr)
+        torch.cuda.synchronize()
+    for first in (True, False):
+        with nhq.Index.create(X, A, CONST) as ix:
+            nhq.nhq_index_set_graph(ix.handle, nbr)
+            cand = torch.empty((w.N, 32), dtype=torch.uint32, device="cuda:0")
+            ids, g, chi = empty_out(w.nq, 10)
+            torch.cuda.synchronize()
+            s1, s2 = torch.cuda.Stream(), torch.cuda.Stream()
+            if first:
+                nhq.nhq_knn(ix.handle, 32, cand, stream=s1)
+            nhq.nhq_search(ix.handle, Qv, QA, 10, 32, ids, g, chi, seed=1,
+                           seed_mode=nhq.SEED_ATTRIBUTE, stream=s2)
+            torch.cuda.synchronize()
+            outs.append((ids_i64(ids), g.cpu().numpy()))
+    assert (outs[0][0] == outs[1][0]).all() and np.array_equal(outs[0][1], outs[1][1])
