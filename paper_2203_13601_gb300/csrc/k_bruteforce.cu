@@ -87,18 +87,6 @@ __device__ __forceinline__ bool rec_less(float ga, uint32_t ia, float gb, uint32
     return ga < gb || (ga == gb && ia < ib);
 }
 
-// A squared distance that every pair with Gamma <= g stays below or equals.  Gamma is at
-// least its vector term in these modes, and sqrt, product and square are each rounded
-// once (relative 2^-24), which the factors cover; the addend covers subnormal results.
-__device__ __forceinline__ float admitted_dist2(float g, const Fusion &w) {
-    float s = INF;
-    if (w.mode == NHQ_W_PROPORTIONAL || w.mode == NHQ_W_FILTER)
-        s = g;
-    else if (w.mode == NHQ_W_CONSTANT && w.wv > 1e-30f)
-        s = (g / w.wv) * 1.00001f;
-    return s * s * 1.00001f + 1e-36f;
-}
-
 // Two differences in one instruction, each rounded as a single one is: six issue slots for
 // four dimensions of a pair instead of eight (candidate sets of 60,000 objects 44.8 ->
 // 41.2 ms, filter truth of 10,000 queries 1.79 -> 1.65 ms).  The sums stay one chain.

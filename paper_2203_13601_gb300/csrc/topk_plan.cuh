@@ -22,6 +22,21 @@ __host__ __device__ inline uint64_t claimed_units(unsigned long long at) {
     return at & ((1ull << kUnitBits) - 1);
 }
 
+// A squared distance that every pair with Gamma <= g stays below or equals.  Gamma is at
+// least its vector term in these modes, and sqrt, product and square are each rounded once
+// (relative 2^-24), which the factors cover; the addend covers squares below the normal
+// range.  A subnormal product w_v delta has no such relative bound: below 1e-37 nothing is
+// ruled out, unless w_v >= 1e-6, where every nonzero delta (at least 3.7e-23, the root of the
+// smallest squared distance) has a normal product and g stands for delta = 0.
+__host__ __device__ inline float admitted_dist2(float g, const Fusion &w) {
+    float s = __builtin_huge_valf();
+    if (w.mode == NHQ_W_PROPORTIONAL || w.mode == NHQ_W_FILTER)
+        s = g;
+    else if (w.mode == NHQ_W_CONSTANT && w.wv > 1e-30f && (g >= 1e-37f || w.wv >= 1e-6f))
+        s = (g / w.wv) * 1.00001f;
+    return s * s * 1.00001f + 1e-36f;
+}
+
 constexpr int MAX_SLICES = 128;
 
 // Objects per slice of a tuple's run.  Few queries hardly share tuples: short slices, so

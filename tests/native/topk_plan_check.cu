@@ -1,7 +1,9 @@
 // Host-side checks of the exact top-k's plan arithmetic (topk_plan.cuh).  The first
 // argument picks the check; prints "ok" or the first failing case.
+#include <cmath>
 #include <cstdio>
 #include <cstring>
+#include <random>
 
 #include "topk_plan.cuh"
 
@@ -50,12 +52,46 @@ static int check_rows() {
     return 0;
 }
 
+// Gamma of a matching pair (every other one is larger), each operation rounded once
+static float gamma_of(float d2, const Fusion &w) {
+    const volatile float delta = std::sqrt(d2);
+    const volatile float g = w.mode == NHQ_W_CONSTANT ? w.wv * delta : delta;
+    return g;
+}
+
+// no pair that may enter is above the admitted squared distance of the k-th record
+static int check_admitted() {
+    std::mt19937_64 rng(11);
+    auto logu = [&](double lo, double hi) {
+        return (float)std::exp2(std::uniform_real_distribution<double>(lo, hi)(rng));
+    };
+    Fusion w{};
+    for (int trial = 0; trial < 4000000; ++trial) {
+        w.mode = trial % 3 == 0 ? NHQ_W_PROPORTIONAL : trial % 3 == 1 ? NHQ_W_FILTER
+                                                                      : NHQ_W_CONSTANT;
+        w.wv = trial % 2 ? logu(-148, -90) : logu(-30, 30);
+        const float a = trial % 5 == 0 ? 0.f : logu(-149, 100);
+        float b = trial % 7 == 0 ? logu(-149, 100) : a * logu(-1, 1);
+        if (trial == 5) {  // both round to the same Gamma, 2 x 2^-149
+            w.wv = 2e-30f, w.mode = NHQ_W_CONSTANT;
+            b = 2.4e-15f * 2.4e-15f;
+        }
+        const float kth = trial == 5 ? 2.0e-15f * 2.0e-15f : a;
+        const float g = gamma_of(kth, w);
+        if (gamma_of(b, w) <= g && !(b <= admitted_dist2(g, w)))
+            return std::printf("FAIL mode %d w_v %g kth %g other %g\n", w.mode, w.wv, kth, b), 1;
+    }
+    return 0;
+}
+
 int main(int argc, char **argv) {
     int bad = 2;
     if (argc > 1 && !std::strcmp(argv[1], "claims"))
         bad = check_claims();
     else if (argc > 1 && !std::strcmp(argv[1], "rows"))
         bad = check_rows();
+    else if (argc > 1 && !std::strcmp(argv[1], "admitted"))
+        bad = check_admitted();
     if (bad == 0)
         std::printf("ok\n");
     return bad;
