@@ -560,9 +560,12 @@ __device__ __forceinline__ void plan_lookup(const TopkArgs &a, const RunPlan &p,
     p.len[q] = (uint32_t)(h - l);
     if (h == l)
         return;
-    uint32_t s = ((uint32_t)l * 0x9E3779B1u) & p.tmask;
+    uint32_t s = table_slot((uint32_t)l, p.tmask);
     for (uint32_t probe = 0; probe <= p.tmask; ++probe) {  // half empty: ends
-        const uint32_t x = atomicCAS(&p.key[s], 0u, (uint32_t)l + 1u);
+        // a key stays once it is set, so only an empty slot needs the exchange
+        uint32_t x = *reinterpret_cast<const volatile uint32_t *>(&p.key[s]);
+        if (x == 0u)
+            x = atomicCAS(&p.key[s], 0u, (uint32_t)l + 1u);
         if (x == 0u || x == (uint32_t)l + 1u)
             break;
         s = (s + 1) & p.tmask;

@@ -4,6 +4,7 @@
 #include <cstdio>
 #include <cstring>
 #include <random>
+#include <vector>
 
 #include "topk_plan.cuh"
 
@@ -84,6 +85,30 @@ static int check_admitted() {
     return 0;
 }
 
+// equal runs of `len` objects (and of lengths that multiplicative hashes dislike) spread over
+// the table: at half load a random placement probes 1.5 slots on average
+static int check_table() {
+    for (uint32_t len : {1u, 16u, 256u, 1000u, 4096u, 46368u, 65536u, 1u << 20})
+        for (uint32_t slots : {64u, 4096u, 65536u}) {
+            const uint32_t tmask = slots - 1, keys = slots / 2;
+            std::vector<char> used(slots, 0);
+            uint64_t probes = 0, worst = 0, n = 0;
+            for (uint32_t i = 0; i < keys && (uint64_t)i * len < 0x7FFFFFFEu; ++i, ++n) {
+                uint32_t s = table_slot(i * len, tmask);
+                uint64_t p = 1;
+                for (; used[s]; s = (s + 1) & tmask)
+                    ++p;
+                used[s] = 1;
+                probes += p;
+                worst = p > worst ? p : worst;
+            }
+            if (probes > 3 * n || worst > 100)
+                return std::printf("FAIL len=%u slots=%u probes=%.1f worst=%d\n", len, slots,
+                                   (double)probes / n, (int)worst), 1;
+        }
+    return 0;
+}
+
 int main(int argc, char **argv) {
     int bad = 2;
     if (argc > 1 && !std::strcmp(argv[1], "claims"))
@@ -92,6 +117,8 @@ int main(int argc, char **argv) {
         bad = check_rows();
     else if (argc > 1 && !std::strcmp(argv[1], "admitted"))
         bad = check_admitted();
+    else if (argc > 1 && !std::strcmp(argv[1], "table"))
+        bad = check_table();
     if (bad == 0)
         std::printf("ok\n");
     return bad;

@@ -24,7 +24,7 @@ def exe(tmp_path_factory):
     return out
 
 
-@pytest.mark.parametrize("check", ["claims", "rows", "admitted"])
+@pytest.mark.parametrize("check", ["claims", "rows", "admitted", "table"])
 def test_plan_arithmetic(exe, check):
     out = subprocess.run([exe, check], capture_output=True, text=True, timeout=120)
     assert out.returncode == 0, out.stdout + out.stderr
