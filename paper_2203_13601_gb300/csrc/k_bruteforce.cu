@@ -50,6 +50,7 @@ constexpr unsigned long long NO_RECORD = (0x7F800000ull << 32) | kNone;  // (inf
 template <int TY_, int QI_, int CTAS_>
 struct Shape {
     static constexpr int TY = TY_, QI = QI_, TX = NT / TY_, TQ = TY_ * QI_, OJ = TN / TX;
+    static_assert(TX == 16 || TX == 64, "the masks of a tile's pairs are written per warp");
     static constexpr int CTAS = CTAS_;
     static constexpr int QW = (TQ + 7) / 8;  // queries whose lists a warp keeps
 };
@@ -294,18 +295,32 @@ __device__ __forceinline__ void scan_objects(const TopkArgs &a, Smem<T> &sm,
         }
         float(*const D2)[TN] = sm.st[buf ^ 1].D2;
         if (__syncthreads_or(any)) {
-            if (any) {
+            if (__any_sync(FULL, any)) {
 #pragma unroll
                 for (int i = 0; i < T::QI; ++i) {
                     const int r = ty + T::TY * i;
                     const float t2 = sm.t2[r];
+                    unsigned m[T::OJ];
 #pragma unroll
-                    for (int j = 0; j < T::OJ; ++j)
-                        if (acc[i][j] <= t2) {
-                            const int c = tx + T::TX * j;
-                            D2[r][c] = acc[i][j];
-                            atomicOr(&sm.mask[r][c >> 5], 1u << (c & 31));
-                        }
+                    for (int j = 0; j < T::OJ; ++j) {
+                        const bool pass = acc[i][j] <= t2;
+                        if (pass)
+                            D2[r][tx + T::TX * j] = acc[i][j];
+                        m[j] = __ballot_sync(FULL, pass);
+                    }
+                    if (T::TX == 16) {  // two rows a warp: 16 columns of each in a ballot
+                        const int half = lane & 16;
+#pragma unroll
+                        for (int j = 0; j < T::OJ; j += 2)
+                            if ((lane & 15) == j / 2)
+                                sm.mask[r][j / 2] = __byte_perm(m[j] >> half, m[j + 1] >> half,
+                                                                0x5410);
+                    } else {  // half a row a warp
+#pragma unroll
+                        for (int j = 0; j < T::OJ; ++j)
+                            if (lane == j)
+                                sm.mask[r][(warp & 1) + 2 * j] = m[j];
+                    }
                 }
             }
             __syncthreads();
