@@ -184,7 +184,7 @@ __device__ __forceinline__ void scan_objects(const TopkArgs &a, Smem<T> &sm,
         sm.cnt[r] = 0;
         sm.tg[r] = INF;
         sm.ti[r] = kNone;
-        sm.t2[r] = INF;
+        sm.t2[r] = sm.q[r] == kNone ? -1.f : INF;  // idle rows: no pair passes
 #pragma unroll
         for (int j = 0; j < 4; ++j)
             sm.mask[r][j] = 0;
@@ -324,38 +324,52 @@ __device__ __forceinline__ void scan_objects(const TopkArgs &a, Smem<T> &sm,
                 }
             }
             __syncthreads();
-            // warp w keeps the lists of queries QW w .. QW w + QW - 1
+            // warp w keeps the lists of queries QW w .. QW w + QW - 1; a lane finishes column
+            // lane of each 32, whose word (or id) it reads once for all of them
+            const int r0 = warp * T::QW;
+            const uint32_t mine = lane < 4 * T::QW && r0 + lane / 4 < T::TQ
+                                      ? sm.mask[r0 + lane / 4][lane & 3]
+                                      : 0u;
+            const unsigned rows = __ballot_sync(FULL, mine != 0);
+            uint32_t col[4];
+            if (rows != 0) {
+#pragma unroll
+                for (int w = 0; w < 4; ++w) {
+                    const uint32_t p = n0 + 32 * w + lane;
+                    col[w] = p < end ? (RUN ? perm[p] : a.attr[p]) : 0u;
+                }
+            }
 #pragma unroll 1
-            for (int r = warp * T::QW; r < min(warp * T::QW + T::QW, T::TQ); ++r) {
-                const uint32_t mine = lane < 4 ? sm.mask[r][lane] : 0u;
-                const uint32_t q = sm.q[r];
-                if (__ballot_sync(FULL, mine != 0) == 0)
+            for (int i = 0; i < T::QW; ++i) {
+                if (((rows >> (4 * i)) & 15u) == 0)
                     continue;
+                const int r = r0 + i;
+                const uint32_t q = sm.q[r];
                 unsigned long long *L = lists + r * k;
                 const float tg = sm.tg[r];
                 const uint32_t ti = sm.ti[r];
                 int cnt = sm.cnt[r];
 #pragma unroll 1
                 for (int w = 0; w < 4; ++w) {
-                    const unsigned m = __shfl_sync(FULL, mine, w);
+                    const unsigned m = __shfl_sync(FULL, mine, 4 * i + w);
+                    if (m == 0)
+                        continue;
                     const uint32_t p = n0 + 32 * w + lane;
+                    const uint32_t cw = w < 2 ? (w == 0 ? col[0] : col[1])
+                                              : (w == 2 ? col[2] : col[3]);
                     unsigned long long c = ~0ull;
-                    if (((m >> lane) & 1u) && p < end && q != kNone) {
-                        const uint32_t id = RUN ? perm[p] : p;
+                    if (((m >> lane) & 1u) && p < end) {
+                        const uint32_t id = RUN ? cw : p;
                         if (!(a.exclude_self && id == q)) {
-                            const int chi =
-                                RUN ? 0 : chi_packed(sm.qa[r], a.attr[p], sm.qh[r], a.w.lo);
+                            const int chi = RUN ? 0 : chi_packed(sm.qa[r], cw, sm.qh[r], a.w.lo);
                             const float g =
                                 fusion_gamma(__fsqrt_rn(D2[r][32 * w + lane]), chi, a.w);
                             if (g < INF && rec_less(g, id, tg, ti))
                                 c = ((unsigned long long)__float_as_uint(g) << 32) | id;
                         }
                     }
-                    if (m != 0)
-                        list_merge(L, cnt, k, c, sm.cand[warp], lane);
+                    list_merge(L, cnt, k, c, sm.cand[warp], lane);
                 }
-                if (lane < 4)
-                    sm.mask[r][lane] = 0;
                 if (lane == 0)
                     sm.cnt[r] = cnt;
                 if (lane == 0 && cnt == k) {
@@ -370,6 +384,8 @@ __device__ __forceinline__ void scan_objects(const TopkArgs &a, Smem<T> &sm,
                     }
                 }
             }
+            if (mine != 0)
+                sm.mask[r0 + lane / 4][lane & 3] = 0;
             __syncthreads();
         }
 #pragma unroll
