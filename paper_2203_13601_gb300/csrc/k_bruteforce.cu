@@ -538,7 +538,7 @@ __global__ void scan_merge_kernel(TopkArgs a, ScanQueries sq, int tq,
 // run), query slots and list rows in single additions.
 struct RunHeader {
     unsigned long long groups_units;  // see plan_claim
-    unsigned long long list_rows;
+    unsigned long long asked, list_rows;  // of the lists: asked for, handed out
     unsigned slots, left, next;
 };
 struct RunGroup {
@@ -562,6 +562,7 @@ struct RunPlan {
     const uint8_t *codes;  // query attributes, or null: the words are given
     uint32_t *words;
     int tq, slice;  // queries per unit, objects per slice aimed at
+    int busy;       // tiles of queries that fill the chip
 };
 
 __device__ __forceinline__ int64_t lower_bound_word(const uint32_t *a, int64_t n, uint32_t x) {
@@ -576,7 +577,8 @@ __device__ __forceinline__ int64_t lower_bound_word(const uint32_t *a, int64_t n
     return lo;
 }
 
-__device__ __forceinline__ void plan_lookup(const TopkArgs &a, const RunPlan &p, int64_t q) {
+// returns the list rows that the query's run would take
+__device__ __forceinline__ unsigned plan_lookup(const TopkArgs &a, const RunPlan &p, int64_t q) {
     uint32_t word, hi;
     if (p.codes != nullptr) {
         word = pack_query_word(p.codes + q * a.w.m, a.w, &hi);
@@ -590,7 +592,7 @@ __device__ __forceinline__ void plan_lookup(const TopkArgs &a, const RunPlan &p,
     p.lo[q] = (uint32_t)l;
     p.len[q] = (uint32_t)(h - l);
     if (h == l)
-        return;
+        return 0;
     uint32_t s = table_slot((uint32_t)l, p.tmask);
     for (uint32_t probe = 0; probe <= p.tmask; ++probe) {  // half empty: ends
         // a key stays once it is set, so only an empty slot needs the exchange
@@ -603,6 +605,15 @@ __device__ __forceinline__ void plan_lookup(const TopkArgs &a, const RunPlan &p,
     }
     p.home[q] = s;
     p.rank[q] = atomicAdd(&p.tcnt[s], 1u);
+    const unsigned want = (unsigned)run_slices(h - l, p.slice);
+    return want > 1 ? want : 0;
+}
+
+// adds up what a warp's queries ask for
+__device__ __forceinline__ void plan_ask(const RunPlan &p, unsigned mine) {
+    const unsigned sum = __reduce_add_sync(FULL, mine);
+    if ((threadIdx.x & 31) == 0 && sum > 0)
+        atomicAdd(&p.hdr->asked, (unsigned long long)sum);
 }
 
 __device__ __forceinline__ void plan_group(const RunPlan &p, int64_t q) {
@@ -613,14 +624,14 @@ __device__ __forceinline__ void plan_group(const RunPlan &p, int64_t q) {
     g.len = p.len[q];
     g.cnt = p.tcnt[p.home[q]];
     g.base = atomicAdd(&p.hdr->slots, g.cnt);
-    int64_t s = run_slices(g.len, p.slice);
-    g.lbase = 0;
-    if (s > 1) {
-        g.lbase = atomicAdd(&p.hdr->list_rows, (unsigned long long)g.cnt * s);
-        s = slices_with_room(s, g.cnt, g.lbase, p.rows);
-    }
+    const int64_t tiles = (g.cnt + p.tq - 1) / p.tq;
+    const int64_t s =
+        granted_slices(run_slices(g.len, p.slice), tiles,
+                       *reinterpret_cast<const volatile unsigned long long *>(&p.hdr->asked),
+                       p.rows, p.busy);
+    g.lbase = s > 1 ? atomicAdd(&p.hdr->list_rows, (unsigned long long)g.cnt * s) : 0;
     g.slices = (int)s;
-    const unsigned long long units = (unsigned long long)((g.cnt + p.tq - 1) / p.tq) * s;
+    const unsigned long long units = (unsigned long long)tiles * s;
     const unsigned long long at = atomicAdd(&p.hdr->groups_units, plan_claim(units));
     g.ubase = claimed_units(at);
     g.pad = 0;
@@ -635,9 +646,11 @@ __device__ __forceinline__ void plan_slot(const RunPlan &p, int64_t q) {
 }
 
 __global__ void run_lookup_kernel(TopkArgs a, RunPlan p) {
+    unsigned asked = 0;
     for (int64_t q = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; q < a.nq;
          q += (int64_t)gridDim.x * blockDim.x)
-        plan_lookup(a, p, q);
+        asked += plan_lookup(a, p, q);
+    plan_ask(p, asked);
 }
 __global__ void run_group_kernel(TopkArgs a, RunPlan p) {
     for (int64_t q = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; q < a.nq;
@@ -656,8 +669,10 @@ __global__ void __launch_bounds__(1024) run_plan_kernel(TopkArgs a, RunPlan p) {
     for (uint32_t t = threadIdx.x; t <= p.tmask; t += blockDim.x)
         p.key[t] = p.tcnt[t] = 0u;
     __syncthreads();
+    unsigned asked = 0;
     for (int64_t q = threadIdx.x; q < a.nq; q += blockDim.x)
-        plan_lookup(a, p, q);
+        asked += plan_lookup(a, p, q);
+    plan_ask(p, asked);
     __syncthreads();
     for (int64_t q = threadIdx.x; q < a.nq; q += blockDim.x)
         plan_group(p, q);
@@ -965,6 +980,8 @@ cudaError_t launch_topk_runs(const TopkArgs &args, const uint8_t *codes,
     const bool few = a.nq <= 64;
     p.tq = few ? Narrow::TQ : Mid::TQ;
     p.slice = run_slice_length(a.nq);
+    const int ctas = few ? resident_ctas<Narrow>(a.k, sm_count) : resident_ctas<Mid>(a.k, sm_count);
+    p.busy = 2 * ctas;
     cudaError_t e;
     if (a.nq <= 2048) {
         run_plan_kernel<<<1, a.nq <= 256 ? 256 : 1024, 0, s>>>(a, p);
@@ -981,8 +998,7 @@ cudaError_t launch_topk_runs(const TopkArgs &args, const uint8_t *codes,
         if ((e = cudaGetLastError()) != cudaSuccess)
             return e;
     }
-    e = few ? launch_runs<Narrow>(a, p, resident_ctas<Narrow>(a.k, sm_count), s)
-            : launch_runs<Mid>(a, p, resident_ctas<Mid>(a.k, sm_count), s);
+    e = few ? launch_runs<Narrow>(a, p, ctas, s) : launch_runs<Mid>(a, p, ctas, s);
     if (e != cudaSuccess)
         return e;
     const int64_t mb = (a.nq + 7) / 8;

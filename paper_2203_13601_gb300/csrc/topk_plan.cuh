@@ -63,29 +63,35 @@ __host__ __device__ inline int64_t run_slices(int64_t len, int slice) {
 
 // Rows of k records kept for the lists of sliced runs: none where no run can take two
 // slices, never more than nq queries on the longest run could use, six for each query
-// (10,000 queries over a million objects of 600 tuples use five) or twelve tiles for each
-// SM, and at most 128 MB, since the index keeps them: 10,000 queries take 48 MB at k = 100
-// and 123 MB at k = 256.  (While neither N nor the bytes counted: 266 and 680 MB, and 658 MB
-// for 5,000 at k = 256 over 1,300 objects, which use none.  64 MB would cost the 10,000 at
+// (10,000 queries over a million objects of 600 tuples use five) or 24 tiles for each SM,
+// and at most 128 MB, since the index keeps them: 10,000 queries take 93 MB at k = 100 and
+// 134 MB at k = 256.  (While neither N nor the bytes counted: 266 and 680 MB, and 658 MB for
+// 5,000 at k = 256 over 1,300 objects, which use none.  64 MB would cost the 10,000 at
 // k = 256 half their speed: 8.2 ms instead of 4.2.)
 constexpr size_t kRunListBytes = size_t(128) << 20;
 inline int64_t run_list_rows(int64_t nq, int64_t N, int k, int sm_count) {
     const int64_t most = run_slices(N, run_slice_length(nq));
     if (most == 1)
         return 0;
-    const int64_t fill = 12 * (int64_t)sm_count * 32;
+    const int64_t fill = 24 * (int64_t)sm_count * 32;
     int64_t rows = 6 * nq > fill ? 6 * nq : fill;
     rows = rows < nq * most ? rows : nq * most;
     const int64_t fit = (int64_t)(kRunListBytes / ((sizeof(uint32_t) + sizeof(float)) * k));
     return rows < fit ? rows : fit;
 }
 
-// Slices of a run that wants `want` of them for cnt queries and claimed cnt * want list
-// rows from `base` on, when there are `rows`: as many as fit; one slice needs no row.
-__host__ __device__ inline int64_t slices_with_room(int64_t want, int64_t cnt, uint64_t base,
-                                                    int64_t rows) {
-    const int64_t fit = base < (uint64_t)rows ? (rows - (int64_t)base) / cnt : 0;
-    const int64_t s = want < fit ? want : fit;
+// Slices of a run that would take `want` of them for `tiles` tiles of queries, where the
+// queries of all sliced runs ask for `all` list rows and there are `rows`: every run gives
+// up the same share, so that none is left with one slice while others have many (whoever
+// came first took all before: 2,000 queries over 100,000 objects of two tuples, k = 100,
+// 2.5 ms instead of 2.2), and the rows handed out stay within `rows`.  A run of `busy` tiles
+// fills the chip by itself and takes one slice: more would only add lists (candidate sets
+// of 30,000 objects of one tuple, 938 tiles: 10.8 ms, 13.2 with six slices).
+__host__ __device__ inline int64_t granted_slices(int64_t want, int64_t tiles, uint64_t all,
+                                                  int64_t rows, int busy) {
+    if (tiles >= busy)
+        return 1;
+    const int64_t s = all > (uint64_t)rows ? (int64_t)((uint64_t)want * rows / all) : want;
     return s > 1 ? s : 1;
 }
 

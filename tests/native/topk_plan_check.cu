@@ -40,12 +40,27 @@ static int check_rows() {
                 const int64_t most = run_slices(N, run_slice_length(nq));
                 bool ok = rows >= 0 && rows <= nq * most && rows * 8 * k <= (128 << 20);
                 ok = ok && (most > 1 || rows == 0);
-                uint64_t base = 0;  // groups of ever more queries on the longest run
-                for (int64_t cnt = 1; cnt <= nq && ok; cnt = cnt * 3 + 1) {
-                    const int64_t s = slices_with_room(most, cnt, base, rows);
-                    ok = s >= 1 && s <= most && (s == 1 || (int64_t)base + s * cnt <= rows);
-                    base += (uint64_t)(cnt * most);
+                // groups of ever more queries on ever shorter runs, of one query and more
+                uint64_t all = 0, out = 0;
+                for (int pass = 0; pass < 2; ++pass) {
+                    int64_t left = nq, len = N;
+                    for (int64_t cnt = 1; left > 0; cnt = cnt * 3 + 1, len = len * 2 / 3 + 1) {
+                        const int64_t n = cnt < left ? cnt : left;
+                        const int64_t want = run_slices(len, run_slice_length(nq));
+                        left -= n;
+                        if (want < 2)
+                            continue;
+                        if (pass == 0) {
+                            all += (uint64_t)(n * want);
+                            continue;
+                        }
+                        const int64_t s = granted_slices(want, (n + 31) / 32, all, rows, 912);
+                        ok = ok && s >= 1 && s <= want && (all > (uint64_t)rows || s == want ||
+                                                           (n + 31) / 32 >= 912);
+                        out += s > 1 ? (uint64_t)(n * s) : 0;
+                    }
                 }
+                ok = ok && out <= (uint64_t)rows;
                 if (!ok)
                     return std::printf("FAIL nq=%lld N=%lld k=%d rows=%lld\n", (long long)nq,
                                        (long long)N, k, (long long)rows), 1;

@@ -77,12 +77,12 @@ def _free():
     return torch.cuda.mem_get_info()[0]
 
 
-# rows of the lists: none (no run reaches two slices), then 48 and 123 MB, beside the plan's
+# rows of the lists: none (no run reaches two slices), then 89 and 128 MB, beside the plan's
 # tables of about 1 MB and, under constant weights, the lists of the queries that are left
 # for the scan (at most 20 MB); allocations come in 2 MB pages
 @pytest.mark.parametrize("N,nq,k,weights,limit", [
-    (1300, 5000, 256, "filter", 8), (60000, 10000, 100, "filter", 56),
-    (60000, 10000, 100, CONST, 80), (60000, 10000, 256, CONST, 152)])
+    (1300, 5000, 256, "filter", 8), (60000, 10000, 100, "filter", 96),
+    (60000, 10000, 100, CONST, 116), (60000, 10000, 256, CONST, 152)])
 def test_working_memory_of_an_exact_batch(nhq, warm, N, nq, k, weights, limit):
     w = synth.int_valued(N, nq, 32, cards=(2, 3), n_comp=9, seed=N)
     with nhq.Index.create(dev(w.X), dev(w.A), CONST) as ix:
@@ -96,7 +96,7 @@ def test_working_memory_of_an_exact_batch(nhq, warm, N, nq, k, weights, limit):
 
 
 def test_runs_short_of_list_rows_take_fewer_slices(nhq):
-    # k = 256: 58,368 rows; one tuple asks for 4,000 x 44, small ones beside it
+    # k = 256: 65,536 rows; one tuple asks for 4,000 x 45, small ones beside it
     rng = np.random.default_rng(4)
     w = synth.int_valued(100000, 4400, 12, cards=(2, 3, 4), n_comp=9, seed=9)
     often = rng.random(w.N) < 0.9
