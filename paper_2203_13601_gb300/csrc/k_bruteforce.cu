@@ -18,7 +18,8 @@
 // tuple's run of the attribute order, and a query whose k-th record there is below
 // Gamma(delta = 0, chi = 1) is finished: Gamma does not fall as delta or chi grows, so no
 // other object can enter.  The queries for which that fails (constant weights only) go
-// through the full scan afterwards, counted on the device.
+// through the full scan afterwards, counted on the device; a long run that is going to fail
+// is given up early.
 //
 // What bounds it: the full scan the FP32 pipe and the issue slots around it.  Candidate
 // sets of 60,000 objects (d = 96, K = 64, proportional weights) take 41.2 ms, half the FP32
@@ -41,6 +42,7 @@ constexpr int TN = 128;     // objects per tile
 constexpr int DC = 32;      // dimensions per staged chunk
 constexpr int DS = DC + 4;  // staged row stride: 16-byte aligned rows, read as float4
 constexpr int NT = 256;     // threads per CTA
+constexpr uint32_t PROBE = 512;  // objects (k <= 256) after which a long run is judged
 constexpr unsigned FULL = 0xFFFFFFFFu;
 constexpr float INF = __builtin_huge_valf();
 constexpr unsigned long long NO_RECORD = (0x7F800000ull << 32) | kNone;  // (inf, none)
@@ -169,12 +171,14 @@ __device__ __forceinline__ void list_merge(unsigned long long *L, int &cnt, int 
 // given, holds for each query the smallest k-th Gamma that any slice has reached (as
 // bits): a record above it is in no final list, so every slice stops inserting what
 // another one already rules out.  Every thread of the CTA calls it with the same arguments.
+// until > 0 (RUN): gives up, returning false, where after PROBE objects more than half of the
+// tile's queries have no k records below it.
 template <class T, bool RUN>
-__device__ __forceinline__ void scan_objects(const TopkArgs &a, Smem<T> &sm,
+__device__ __forceinline__ bool scan_objects(const TopkArgs &a, Smem<T> &sm,
                                              unsigned long long *lists, uint32_t begin,
                                              uint32_t end,
                                              const uint32_t *__restrict__ perm,
-                                             uint32_t *kth) {
+                                             uint32_t *kth, float until) {
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int ty = tid / T::TX, tx = tid % T::TX;
     const int k = a.k;
@@ -235,7 +239,16 @@ __device__ __forceinline__ void scan_objects(const TopkArgs &a, Smem<T> &sm,
         kth != nullptr && tid < T::TQ && sm.q[tid] != kNone ? kth + sm.q[tid] : nullptr;
     uint32_t seen = ~0u;
     int buf = 0;
+    bool done = true;
     for (uint32_t n0 = begin; n0 < end; n0 += TN) {  // N < 2^31: no overflow
+        if (RUN && until > 0.f && n0 == begin + PROBE) {
+            const bool mine = tid < T::TQ && sm.q[tid] != kNone;
+            const int open = __syncthreads_count(mine && !(sm.tg[tid] < until));
+            if (2 * open > __syncthreads_count(mine)) {
+                done = false;
+                break;
+            }
+        }
         rows_of(n0 + TN, nrow);
         if (watch != nullptr) {
             if (seen < __float_as_uint(sm.tg[tid])) {
@@ -393,6 +406,7 @@ __device__ __forceinline__ void scan_objects(const TopkArgs &a, Smem<T> &sm,
             row[i] = nrow[i];
     }
     asm volatile("cp.async.wait_group 0;" ::: "memory");
+    return done;
 }
 
 // the final row of query q: record e is (g, id) for e < k
@@ -453,7 +467,7 @@ __global__ void __launch_bounds__(NT, T::CTAS) scan_kernel(TopkArgs a, ScanQueri
         const int64_t begin = split * per;
         const int64_t end = a.N < begin + per ? a.N : begin + per;
         scan_objects<T, false>(a, sm, lists, (uint32_t)(begin < end ? begin : end),
-                               (uint32_t)end, nullptr, S > 1 ? sq.kth : nullptr);
+                               (uint32_t)end, nullptr, S > 1 ? sq.kth : nullptr, 0.f);
         for (int r = warp * T::QW; r < min(warp * T::QW + T::QW, T::TQ); ++r) {
             if (sm.q[r] == kNone)
                 continue;
@@ -549,6 +563,7 @@ struct RunGroup {
 };
 struct RunPlan {
     RunHeader *hdr;
+    uint32_t *failed;  // [nq] queries that a long run was given up for (constant weights)
     uint32_t *key, *tcnt, *tgroup;  // [T] run start + 1, queries, group
     uint32_t tmask;
     uint32_t *lo, *len, *home, *rank;  // [nq]
@@ -668,6 +683,8 @@ __global__ void __launch_bounds__(1024) run_plan_kernel(TopkArgs a, RunPlan p) {
         *p.hdr = RunHeader{};
     for (uint32_t t = threadIdx.x; t <= p.tmask; t += blockDim.x)
         p.key[t] = p.tcnt[t] = 0u;
+    for (int64_t q = threadIdx.x; q < a.nq; q += blockDim.x)
+        p.failed[q] = 0u;
     __syncthreads();
     unsigned asked = 0;
     for (int64_t q = threadIdx.x; q < a.nq; q += blockDim.x)
@@ -682,6 +699,11 @@ __global__ void __launch_bounds__(1024) run_plan_kernel(TopkArgs a, RunPlan p) {
 }
 
 // Units of the plan, taken from a counter (runs differ in length by orders of magnitude).
+// Under constant weights a run of more than a quarter of all objects is judged early: where
+// omega_l does not exceed the vector term, the scan answers its queries anyway, and the run
+// would have cost up to as much again (candidate sets of 30,000 objects of two tuples,
+// w_l = 0.01: 18.5 ms, judged 12.9; the scan alone 11.4).  A run of all objects needs no
+// scan afterwards (one tuple: 21.6 ms, now 10.5).
 template <class T>
 __global__ void __launch_bounds__(NT, T::CTAS) run_kernel(TopkArgs a, RunPlan p) {
     extern __shared__ __align__(16) unsigned char smem[];
@@ -710,18 +732,32 @@ __global__ void __launch_bounds__(NT, T::CTAS) run_kernel(TopkArgs a, RunPlan p)
         const RunGroup g = p.group[l];
         const int v = (int)(u - (int64_t)g.ubase);
         const int tile = v / g.slices, split = v % g.slices;
+        const float until = a.w.mode == NHQ_W_CONSTANT && g.len < a.N && g.len > a.N / 4
+                                ? fusion_gamma(0.f, 1, a.w)
+                                : 0.f;
+        bool wanted = until == 0.f;
         for (int r = tid; r < T::TQ; r += NT) {
             const uint32_t i = (uint32_t)tile * T::TQ + r;
-            sm.q[r] = i < g.cnt ? p.slot[g.base + i] : kNone;
+            const uint32_t q = i < g.cnt ? p.slot[g.base + i] : kNone;
+            sm.q[r] = q;
+            wanted = wanted ||
+                     (q != kNone &&
+                      *reinterpret_cast<const volatile uint32_t *>(p.failed + q) == 0u);
         }
-        __syncthreads();
+        if (!__syncthreads_or(wanted))
+            continue;  // another slice has given up for all of them
         const int64_t per = (((int64_t)g.len + g.slices - 1) / g.slices + TN - 1) / TN * TN;
         const int64_t run_end = (int64_t)g.lo + g.len;
         int64_t begin = (int64_t)g.lo + split * per;
         begin = begin < run_end ? begin : run_end;
         const int64_t end = begin + per < run_end ? begin + per : run_end;
-        scan_objects<T, true>(a, sm, lists, (uint32_t)begin, (uint32_t)end, p.id_sorted,
-                              nullptr);
+        if (!scan_objects<T, true>(a, sm, lists, (uint32_t)begin, (uint32_t)end, p.id_sorted,
+                                   nullptr, until)) {
+            for (int r = tid; r < T::TQ; r += NT)
+                if (sm.q[r] != kNone && atomicExch(p.failed + sm.q[r], 1u) == 0u)
+                    p.left[atomicAdd(&p.hdr->left, 1u)] = sm.q[r];
+            continue;
+        }
         for (int r = warp * T::QW; r < min(warp * T::QW + T::QW, T::TQ); ++r) {
             if (sm.q[r] == kNone)
                 continue;
@@ -740,7 +776,7 @@ __global__ void __launch_bounds__(NT, T::CTAS) run_kernel(TopkArgs a, RunPlan p)
             }
             if (g.slices > 1)
                 continue;
-            if (lane == 0 && a.w.mode != NHQ_W_FILTER &&
+            if (lane == 0 && a.w.mode != NHQ_W_FILTER && g.len < a.N &&
                 !(cnt == a.k && __uint_as_float((uint32_t)(lists[r * a.k + a.k - 1] >> 32)) <
                                        fusion_gamma(0.f, 1, a.w)))
                 p.left[atomicAdd(&p.hdr->left, 1u)] = sm.q[r];
@@ -760,7 +796,7 @@ __global__ void run_merge_kernel(TopkArgs a, RunPlan p) {
         } else {
             const RunGroup &g = p.group[p.tgroup[p.home[q]]];
             const int S = g.slices;
-            if (S == 1)
+            if (S == 1 || (a.w.mode != NHQ_W_FILTER && p.failed[q] != 0u))
                 continue;
             const int64_t o = ((int64_t)g.lbase + (int64_t)p.rank[q] * S) * a.k;
             merge_lists(p.part_id + o, p.part_g + o, S, a.k, lane,
@@ -770,7 +806,7 @@ __global__ void run_merge_kernel(TopkArgs a, RunPlan p) {
                             last = gm;
                         });
         }
-        if (lane == 0 && a.w.mode != NHQ_W_FILTER && !(last < fusion_gamma(0.f, 1, a.w)))
+        if (lane == 0 && a.w.mode != NHQ_W_FILTER && p.len[q] < a.N && !(last < fusion_gamma(0.f, 1, a.w)))
             p.left[atomicAdd(&p.hdr->left, 1u)] = (uint32_t)q;
     }
 }
@@ -885,7 +921,7 @@ cudaError_t launch_topk(const TopkArgs &a, void *scratch, size_t scratch_bytes, 
 namespace {
 
 struct RunLayout {
-    size_t table, words, query, slot, group, left, part, kth, scan, bytes;
+    size_t failed, table, words, query, slot, group, left, part, kth, scan, bytes;
     uint32_t tmask;
     int64_t rows, srows;
 };
@@ -906,6 +942,7 @@ RunLayout run_layout(const TopkArgs &a, int sm_count) {
         off += (bytes + 255) & ~(size_t)255;
         return at;
     };
+    L.failed = take(sizeof(uint32_t) * (size_t)a.nq);
     L.table = take(3 * sizeof(uint32_t) * (size_t)T);
     L.words = take(sizeof(uint32_t) * (size_t)a.nq);
     L.query = take(4 * sizeof(uint32_t) * (size_t)a.nq);
@@ -956,6 +993,7 @@ cudaError_t launch_topk_runs(const TopkArgs &args, const uint8_t *codes,
     RunPlan p;
     const size_t T = (size_t)L.tmask + 1;
     p.hdr = reinterpret_cast<RunHeader *>(base);
+    p.failed = reinterpret_cast<uint32_t *>(base + L.failed);
     p.key = reinterpret_cast<uint32_t *>(base + L.table);
     p.tcnt = p.key + T;
     p.tgroup = p.tcnt + T;

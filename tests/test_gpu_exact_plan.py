@@ -182,3 +182,19 @@ def test_attribute_order_of_an_exact_call_serves_other_streams(nhq):
             torch.cuda.synchronize()
             outs.append((ids_i64(ids), g.cpu().numpy()))
     assert (outs[0][0] == outs[1][0]).all() and np.array_equal(outs[0][1], outs[1][1])
+
+
+# runs of all objects, of a half and of a third, in one slice and in several, under weights
+# for which none, some or all of the queries are finished by their run: all of them are
+# judged after 512 objects
+@pytest.mark.parametrize("N,nq,k,cards", [(9000, 300, 10, (1,)), (9000, 300, 256, (2,)),
+                                          (24000, 2500, 33, (2,)), (700, 40000, 5, (3,)),
+                                          (20000, 2100, 1, (3,))])
+@pytest.mark.parametrize("wl", [0.01, 60.0, 120.0, 240.0, 10000.0])
+def test_long_runs_under_weak_and_strong_weights(nhq, N, nq, k, cards, wl):
+    w = synth.int_valued(N, nq, 32, cards=cards, n_comp=9, seed=N + nq + k)
+    with nhq.Index.create(dev(w.X), dev(w.A), (1.0, wl)) as ix:
+        nhq.nhq_index_build_cells(ix.handle, 4)  # brings the attribute order
+        ids, g, chi = empty_out(nq, k)
+        nhq.nhq_brute_force(ix.handle, dev(w.Qv), dev(w.QA), k, ids, g, chi)
+        _check(w, k, ids, g, (1.0, wl), np.arange(0, nq, max(1, nq // 300)))
