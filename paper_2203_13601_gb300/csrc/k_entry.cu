@@ -330,7 +330,10 @@ constexpr int SLICE = 128;
 // acc[i][j] (+)= sum over k in [k0, k1) of a(k, ty * 4 + i) b(k, tx * 4 + j), k ascending.
 // AK / BK: the operand is contiguous along k in memory (the staging loop follows it).
 // sum (or null): the threads with ty = 0 also add b(k, tx + 16 j) over k into sum[j].
-template <bool AK, bool BK, class LA, class LB>
+// COMP: the products of 8 k are summed as one chain, four of these as another, and the sums
+// of the chunks with Kahan's compensation.  (One chain over all E cells of a gradient had up
+// to four times the error of 32 strided chains and a tree, which summed them before.)
+template <bool AK, bool BK, bool COMP = false, class LA, class LB>
 __device__ __forceinline__ void tile_product(float acc[4][4], int64_t k0, int64_t k1, LA la, LB lb,
                                              float (*As)[GP], float (*Bs)[GP],
                                              float *sum = nullptr) {
@@ -346,6 +349,7 @@ __device__ __forceinline__ void tile_product(float acc[4][4], int64_t k0, int64_
             rb[i] = kb + kk < k1 ? lb(kb + kk, c) : 0.f;
         }
     };
+    float lost[4][4] = {};  // COMP: what adding to acc has rounded away
     fetch(k0);
     for (int64_t kb = k0; kb < k1; kb += GK) {
 #pragma unroll
@@ -357,6 +361,43 @@ __device__ __forceinline__ void tile_product(float acc[4][4], int64_t k0, int64_
         __syncthreads();
         if (kb + GK < k1)
             fetch(kb + GK);
+        if (COMP) {
+            float chunk[4][4] = {};
+#pragma unroll 2
+            for (int k8 = 0; k8 < GK; k8 += 8) {
+                float p[4][4] = {};
+#pragma unroll
+                for (int kk = 0; kk < 8; ++kk) {
+                    float a[4], b[4];
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) {
+                        a[i] = As[k8 + kk][ty * 4 + i];
+                        b[i] = Bs[k8 + kk][tx + 16 * i];
+                    }
+#pragma unroll
+                    for (int i = 0; i < 4; ++i)
+#pragma unroll
+                        for (int j = 0; j < 4; ++j)
+                            p[i][j] = fmaf(a[i], b[j], p[i][j]);
+                }
+#pragma unroll
+                for (int i = 0; i < 4; ++i)
+#pragma unroll
+                    for (int j = 0; j < 4; ++j)
+                        chunk[i][j] += p[i][j];
+            }
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    const float y = chunk[i][j] - lost[i][j];
+                    const float t = acc[i][j] + y;
+                    lost[i][j] = (t - acc[i][j]) - y;
+                    acc[i][j] = t;
+                }
+            __syncthreads();
+            continue;
+        }
 #pragma unroll 8
         for (int kk = 0; kk < GK; ++kk) {
             float a[4], b[4];
@@ -492,7 +533,7 @@ __global__ void train_softmax_kernel(float *T, const int32_t *__restrict__ y, in
     }
 }
 
-// dZ[b][h] = [H > 0] sum_o dT[b][o] W2[h][o], o ascending; grid (ceil(B/64))
+// dZ[b][h] = [H > 0] sum_o dT[b][o] W2[h][o]; grid (ceil(B/64))
 __global__ void __launch_bounds__(256) train_dz_kernel(const float *__restrict__ P,
                                                        const float *__restrict__ H,
                                                        const float *__restrict__ dT, int B, int E,
@@ -501,7 +542,7 @@ __global__ void __launch_bounds__(256) train_dz_kernel(const float *__restrict__
     const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
     const int b0 = blockIdx.x * GT;
     float acc[4][4] = {};
-    tile_product<true, true>(
+    tile_product<true, true, true>(
         acc, 0, E,
         [&](int64_t k, int r) { return b0 + r < B ? dT[(int64_t)(b0 + r) * E + k] : 0.f; },
         [&](int64_t k, int c) { return P[L.oW2 + (int64_t)c * E + k]; }, As, Bs);
