@@ -487,12 +487,12 @@ __global__ void __launch_bounds__(256) train_out_kernel(const float *__restrict_
     }
 }
 
-// dT = (softmax(T) - onehot(label)) * inv_n per sample (a warp each); loss += (lse - t_y) * inv_n
-// (one addition to it per block of eight samples).
+// dT = (softmax(T) - onehot(label)) * inv_n per sample (a warp each); losses[block] = the sum of
+// (lse - t_y) * inv_n over the block's eight samples.
 // A label outside 0..E-1 contributes nothing.
 // T becomes dT in place (a lane reads the elements that it writes).
 __global__ void train_softmax_kernel(float *T, const int32_t *__restrict__ y, int B, int E,
-                                     float inv_n, float *__restrict__ loss) {
+                                     float inv_n, float *__restrict__ losses) {
     __shared__ float part[8];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int b = blockIdx.x * 8 + warp;
@@ -529,7 +529,7 @@ __global__ void train_softmax_kernel(float *T, const int32_t *__restrict__ y, in
 #pragma unroll
         for (int w = 0; w < 8; ++w)
             sum += part[w];
-        atomicAdd(loss, sum);
+        losses[blockIdx.x] = sum;
     }
 }
 
@@ -597,14 +597,35 @@ __global__ void __launch_bounds__(256) train_gw_kernel(const float *__restrict__
 
 // G += the slices of both gradients: 32 values per block, eight warps summing every
 // eighth slice in order, then the eight sums in order.  W1 | b1 and W2 | b2 are each one
-// run of the parameter vector, laid out as train_gw_kernel lays out its rows.
+// run of the parameter vector, laid out as train_gw_kernel lays out its rows.  The first
+// block adds the softmax's block sums to the loss (as additions to one value, in whatever
+// order, they moved it by 3e-7 of itself between runs).
 __global__ void __launch_bounds__(256) grad_reduce_kernel(const float *__restrict__ part1,
                                                           int64_t n1,
                                                           const float *__restrict__ part2,
                                                           int64_t n2, int slices,
-                                                          float *__restrict__ G) {
+                                                          float *__restrict__ G,
+                                                          const float *__restrict__ losses,
+                                                          int nlosses, float *loss) {
     __shared__ float sums[8][32];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    if (blockIdx.x == 0) {
+        float acc = 0.f;
+        for (int i = threadIdx.x; i < nlosses; i += 256)
+            acc += losses[i];
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1)
+            acc += __shfl_xor_sync(FULL, acc, o);
+        if (lane == 0)
+            sums[0][warp] = acc;
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            for (int w = 1; w < 8; ++w)
+                acc += sums[0][w];
+            *loss += acc;
+        }
+        __syncthreads();
+    }
     for (int64_t i0 = blockIdx.x * (int64_t)32; i0 < n1 + n2; i0 += (int64_t)gridDim.x * 32) {
         const int64_t i = i0 + lane;
         float acc = 0.f;
@@ -769,11 +790,11 @@ int entry_train_chunk(int64_t n, int d, int E) {
     return (int)(n < B ? n : B);
 }
 
-// Working memory of one chunk of B samples: H, dZ [B][64], T [B][E] and the slices' partial
-// sums of (W1 | b1) and (W2 | b2).
+// Working memory of one chunk of B samples: H, dZ [B][64], T [B][E], the slices' partial
+// sums of (W1 | b1) and (W2 | b2) and the losses [ceil(B/8)].
 size_t entry_train_chunk_bytes(int B, int d, int E) {
     const size_t slices = ((size_t)B + SLICE - 1) / SLICE;
-    return sizeof(float) * ((size_t)B * EH * 2 + (size_t)B * E +
+    return sizeof(float) * ((size_t)B * EH * 2 + (size_t)B * E + ((size_t)B + 7) / 8 +
                             slices * ((size_t)(d + 1) * EH + (size_t)(EH + 1) * E)) +
            1024;
 }
@@ -790,6 +811,7 @@ cudaError_t entry_grad_accumulate(const float *P, int d, int E, const float *X,
     float *T = dZ + (size_t)B * EH;
     float *part1 = T + (size_t)B * E;
     float *part2 = part1 + (size_t)((B + SLICE - 1) / SLICE) * n1;
+    float *losses = part2 + (size_t)((B + SLICE - 1) / SLICE) * n2;
     const float inv = 1.f / (float)total;
     const unsigned et = (unsigned)((E + GT - 1) / GT);
     cudaError_t e = cudaSuccess;
@@ -800,14 +822,14 @@ cudaError_t entry_grad_accumulate(const float *P, int d, int E, const float *X,
         const unsigned sl = (unsigned)((nb + SLICE - 1) / SLICE);
         train_hidden_kernel<<<bt, 256, 0, s>>>(P, Xb, nb, d, H, L);
         train_out_kernel<<<dim3(bt, et), 256, 0, s>>>(P, H, nb, E, T, L);
-        train_softmax_kernel<<<(nb + 7) / 8, 256, 0, s>>>(T, y + b0, nb, E, inv, loss);
+        train_softmax_kernel<<<(nb + 7) / 8, 256, 0, s>>>(T, y + b0, nb, E, inv, losses);
         train_gw_kernel<<<dim3(et, EH / GT, sl), 256, 0, s>>>(H, EH, nullptr, T, E, nb,
                                                                     part2);
         train_dz_kernel<<<bt, 256, 0, s>>>(P, H, T, nb, E, dZ, L);
         train_gw_kernel<<<dim3(1, (unsigned)((d + GT - 1) / GT), sl), 256, 0, s>>>(Xb, d, P, dZ, EH,
                                                                               nb, part1);
-        grad_reduce_kernel<<<grid_for(n1 + n2, 32), 256, 0, s>>>(part1, n1, part2, n2, (int)sl,
-                                                                  G);
+        grad_reduce_kernel<<<grid_for(n1 + n2, 32), 256, 0, s>>>(part1, n1, part2, n2, (int)sl, G,
+                                                                 losses, (nb + 7) / 8, loss);
         if ((e = cudaGetLastError()) != cudaSuccess)
             return e;
     }
