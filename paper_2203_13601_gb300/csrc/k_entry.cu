@@ -330,10 +330,13 @@ constexpr int SLICE = 128;
 // acc[i][j] (+)= sum over k in [k0, k1) of a(k, ty * 4 + i) b(k, tx * 4 + j), k ascending.
 // AK / BK: the operand is contiguous along k in memory (the staging loop follows it).
 // sum (or null): the threads with ty = 0 also add b(k, tx + 16 j) over k into sum[j].
-// COMP: the products of 8 k are summed as one chain, four of these as another, and the sums
-// of the chunks with Kahan's compensation.  (One chain over all E cells of a gradient had up
-// to four times the error of 32 strided chains and a tree, which summed them before.)
-template <bool AK, bool BK, bool COMP = false, class LA, class LB>
+// LEVELS: 0 sums all k as one chain; 1 the products of 8 k as one chain, four of these (a
+// chunk) as another and the chunks as a third; 2 also eight chunks apart from the rest.
+// One chain over the E cells of a gradient had up to five times the error of 32 strided
+// chains and a tree, which summed them before; 1 has it times 1.1 up to E = 256, 2 times 0.5
+// from 1,024 on (1 would have 1.25 at 4,096).  At E = 256 a step takes 133.6 us with 0 and
+// 1, 135.7 us with 2 or with Kahan's compensation per chunk.
+template <bool AK, bool BK, int LEVELS = 0, class LA, class LB>
 __device__ __forceinline__ void tile_product(float acc[4][4], int64_t k0, int64_t k1, LA la, LB lb,
                                              float (*As)[GP], float (*Bs)[GP],
                                              float *sum = nullptr) {
@@ -349,7 +352,7 @@ __device__ __forceinline__ void tile_product(float acc[4][4], int64_t k0, int64_
             rb[i] = kb + kk < k1 ? lb(kb + kk, c) : 0.f;
         }
     };
-    float lost[4][4] = {};  // COMP: what adding to acc has rounded away
+    float total[4][4] = {};  // of every eight chunks
     fetch(k0);
     for (int64_t kb = k0; kb < k1; kb += GK) {
 #pragma unroll
@@ -361,7 +364,7 @@ __device__ __forceinline__ void tile_product(float acc[4][4], int64_t k0, int64_
         __syncthreads();
         if (kb + GK < k1)
             fetch(kb + GK);
-        if (COMP) {
+        if (LEVELS > 0) {
             float chunk[4][4] = {};
 #pragma unroll 2
             for (int k8 = 0; k8 < GK; k8 += 8) {
@@ -389,12 +392,17 @@ __device__ __forceinline__ void tile_product(float acc[4][4], int64_t k0, int64_
 #pragma unroll
             for (int i = 0; i < 4; ++i)
 #pragma unroll
-                for (int j = 0; j < 4; ++j) {
-                    const float y = chunk[i][j] - lost[i][j];
-                    const float t = acc[i][j] + y;
-                    lost[i][j] = (t - acc[i][j]) - y;
-                    acc[i][j] = t;
-                }
+                for (int j = 0; j < 4; ++j)
+                    acc[i][j] += chunk[i][j];
+            if (LEVELS > 1 && ((kb - k0) / GK & 7) == 7) {
+#pragma unroll
+                for (int i = 0; i < 4; ++i)
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) {
+                        total[i][j] += acc[i][j];
+                        acc[i][j] = 0.f;
+                    }
+            }
             __syncthreads();
             continue;
         }
@@ -418,6 +426,13 @@ __device__ __forceinline__ void tile_product(float acc[4][4], int64_t k0, int64_
             }
         }
         __syncthreads();
+    }
+    if (LEVELS > 1) {
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+#pragma unroll
+            for (int j = 0; j < 4; ++j)
+                acc[i][j] += total[i][j];
     }
 }
 
@@ -534,6 +549,7 @@ __global__ void train_softmax_kernel(float *T, const int32_t *__restrict__ y, in
 }
 
 // dZ[b][h] = [H > 0] sum_o dT[b][o] W2[h][o]; grid (ceil(B/64))
+template <int LEVELS>
 __global__ void __launch_bounds__(256) train_dz_kernel(const float *__restrict__ P,
                                                        const float *__restrict__ H,
                                                        const float *__restrict__ dT, int B, int E,
@@ -542,7 +558,7 @@ __global__ void __launch_bounds__(256) train_dz_kernel(const float *__restrict__
     const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
     const int b0 = blockIdx.x * GT;
     float acc[4][4] = {};
-    tile_product<true, true, true>(
+    tile_product<true, true, LEVELS>(
         acc, 0, E,
         [&](int64_t k, int r) { return b0 + r < B ? dT[(int64_t)(b0 + r) * E + k] : 0.f; },
         [&](int64_t k, int c) { return P[L.oW2 + (int64_t)c * E + k]; }, As, Bs);
@@ -825,7 +841,10 @@ cudaError_t entry_grad_accumulate(const float *P, int d, int E, const float *X,
         train_softmax_kernel<<<(nb + 7) / 8, 256, 0, s>>>(T, y + b0, nb, E, inv, losses);
         train_gw_kernel<<<dim3(et, EH / GT, sl), 256, 0, s>>>(H, EH, nullptr, T, E, nb,
                                                                     part2);
-        train_dz_kernel<<<bt, 256, 0, s>>>(P, H, T, nb, E, dZ, L);
+        if (E <= 256)
+            train_dz_kernel<1><<<bt, 256, 0, s>>>(P, H, T, nb, E, dZ, L);
+        else
+            train_dz_kernel<2><<<bt, 256, 0, s>>>(P, H, T, nb, E, dZ, L);
         train_gw_kernel<<<dim3(1, (unsigned)((d + GT - 1) / GT), sl), 256, 0, s>>>(Xb, d, P, dZ, EH,
                                                                               nb, part1);
         grad_reduce_kernel<<<grid_for(n1 + n2, 32), 256, 0, s>>>(part1, n1, part2, n2, (int)sl, G,
