@@ -323,9 +323,16 @@ __global__ void entry_to_half_kernel(const float *__restrict__ p, __half *__rest
 // gradients (4 and 2 tiles of outputs) split the samples into slices of SLICE, each
 // writing its own partial sums, which grad_reduce_kernel adds in slice order (no atomics:
 // the gradient is the same in every run).  That step took 2,804 us with one thread per
-// output walking all samples of a 2,048-sample chunk in eight chunks, and takes 133 us.
+// output walking all samples of a 2,048-sample chunk in eight chunks, and takes 130 us.
 constexpr int GT = 64, GK = 32, GP = GT + 1;
 constexpr int SLICE = 128;
+// Up to FEW samples and FEW_OUT outputs a step takes kernels with a thread to an output, and
+// up to FEW_HIDDEN samples that for H.  Steps at d = 128, on them | on the tiles: 32 samples
+// 39.6 | 45.7 us (64 and 256 cells) and 57.5 | 66.7 us (4,096), 128 samples 53.9 | 57.9 and
+// 84.2 | 83.0, 200 samples 64.4 | 59.0 and 107 | 92; H alone takes 2 us off at 1,024 and
+// 2,048 samples (14 at d = 960) and adds 2 to 28 at 4,096.
+constexpr int FEW = 128, FEW_HIDDEN = 2048;
+constexpr int64_t FEW_OUT = 1 << 18;  // samples x cells
 
 // acc[i][j] (+)= sum over k in [k0, k1) of a(k, ty * 4 + i) b(k, tx * 4 + j), k ascending.
 // AK / BK: the operand is contiguous along k in memory (the staging loop follows it).
@@ -547,7 +554,6 @@ __global__ void train_softmax_kernel(float *T, const int32_t *__restrict__ y, in
         losses[blockIdx.x] = sum;
     }
 }
-
 // dZ[b][h] = [H > 0] sum_o dT[b][o] W2[h][o]; grid (ceil(B/64))
 template <int LEVELS>
 __global__ void __launch_bounds__(256) train_dz_kernel(const float *__restrict__ P,
@@ -611,9 +617,9 @@ __global__ void __launch_bounds__(256) train_gw_kernel(const float *__restrict__
     }
 }
 
-// G += the slices of both gradients: 32 values per block, eight warps summing every
+// G = (add: +=) the slices of both gradients: 32 values per block, eight warps summing every
 // eighth slice in order, then the eight sums in order.  W1 | b1 and W2 | b2 are each one
-// run of the parameter vector, laid out as train_gw_kernel lays out its rows.  The first
+// run of the parameter vector, laid out as train_gw_kernel lays out its rows.  The last
 // block adds the softmax's block sums to the loss (as additions to one value, in whatever
 // order, they moved it by 3e-7 of itself between runs).
 __global__ void __launch_bounds__(256) grad_reduce_kernel(const float *__restrict__ part1,
@@ -622,10 +628,10 @@ __global__ void __launch_bounds__(256) grad_reduce_kernel(const float *__restric
                                                           int64_t n2, int slices,
                                                           float *__restrict__ G,
                                                           const float *__restrict__ losses,
-                                                          int nlosses, float *loss) {
+                                                          int nlosses, float *loss, bool add) {
     __shared__ float sums[8][32];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    if (blockIdx.x == 0) {
+    if (blockIdx.x == gridDim.x - 1) {
         float acc = 0.f;
         for (int i = threadIdx.x; i < nlosses; i += 256)
             acc += losses[i];
@@ -638,11 +644,14 @@ __global__ void __launch_bounds__(256) grad_reduce_kernel(const float *__restric
         if (threadIdx.x == 0) {
             for (int w = 1; w < 8; ++w)
                 acc += sums[0][w];
-            *loss += acc;
+            *loss = add ? *loss + acc : acc;
+            if (!add)
+                G[0] = 0.f;  // the input scale is not trained
         }
-        __syncthreads();
+        return;
     }
-    for (int64_t i0 = blockIdx.x * (int64_t)32; i0 < n1 + n2; i0 += (int64_t)gridDim.x * 32) {
+    for (int64_t i0 = blockIdx.x * (int64_t)32; i0 < n1 + n2;
+         i0 += (int64_t)(gridDim.x - 1) * 32) {
         const int64_t i = i0 + lane;
         float acc = 0.f;
         if (i < n1 + n2) {
@@ -658,10 +667,109 @@ __global__ void __launch_bounds__(256) grad_reduce_kernel(const float *__restric
 #pragma unroll
             for (int w = 1; w < 8; ++w)
                 acc += sums[w][lane];
-            G[1 + i] += acc;
+            G[1 + i] = add ? G[1 + i] + acc : acc;
         }
         __syncthreads();
     }
+}
+
+// ---- the same step for few samples ----
+// A tile of 64 samples leaves most of the chip idle where there are not many of them, and
+// walks all of E (or d) in one chain of loads: a step of 32 samples at d = 128, E = 1,024
+// took 105 us on tiles alone and takes 42 with an output to a thread (dZ: to a warp).
+
+// H[b][j] as train_hidden_kernel; 4 samples of 64 units per block
+__global__ void few_hidden_kernel(const float *__restrict__ P, const float *__restrict__ X, int B,
+                                  int d, float *__restrict__ H, EntryLayout L) {
+    const int b = blockIdx.x * 4 + (threadIdx.x >> 6), j = threadIdx.x & 63;
+    if (b >= B)
+        return;
+    const float s = P[0];
+    float z = P[L.oB1 + j];
+    for (int i = 0; i < d; ++i)
+        z = fmaf(P[L.oW1 + (int64_t)i * EH + j], s * X[(int64_t)b * d + i], z);
+    H[(int64_t)b * EH + j] = fmaxf(z, 0.f);
+}
+
+// T[b][o] as train_out_kernel; grid (ceil(E/128), B)
+__global__ void few_out_kernel(const float *__restrict__ P, const float *__restrict__ H, int E,
+                               float *__restrict__ T, EntryLayout L) {
+    __shared__ float h[EH];
+    const int b = blockIdx.y;
+    if (threadIdx.x < EH)
+        h[threadIdx.x] = H[(int64_t)b * EH + threadIdx.x];
+    __syncthreads();
+    const int o = blockIdx.x * blockDim.x + threadIdx.x;
+    if (o >= E)
+        return;
+    float t = P[L.oB2 + o];
+    for (int k = 0; k < EH; ++k)
+        t = fmaf(P[L.oW2 + (int64_t)k * E + o], h[k], t);
+    T[(int64_t)b * E + o] = t;
+}
+
+// dZ[b][h] = [H > 0] sum_o dT[b][o] W2[h][o], a warp per pair (b, h); the first warp also
+// puts the softmax's block sums into the loss, where that is given, and 0 into the input
+// scale's place G[0] (add: adds them to the loss)
+__global__ void few_dz_kernel(const float *__restrict__ P, const float *__restrict__ H,
+                              const float *__restrict__ dT, int B, int E,
+                              float *__restrict__ dZ, EntryLayout L,
+                              const float *__restrict__ losses, int nlosses, float *loss,
+                              float *G, bool add) {
+    const int lane = threadIdx.x & 31;
+    const int64_t pair = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+    if (pair >= (int64_t)B * EH)
+        return;
+    if (pair == 0 && loss != nullptr) {
+        float sum = 0.f;
+        for (int i = lane; i < nlosses; i += 32)
+            sum += losses[i];
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1)
+            sum += __shfl_xor_sync(FULL, sum, o);
+        if (lane == 0) {
+            *loss = add ? *loss + sum : sum;
+            if (!add)
+                G[0] = 0.f;
+        }
+    }
+    const int b = (int)(pair / EH), h = (int)(pair % EH);
+    float acc = 0.f;
+    for (int o = lane; o < E; o += 32)
+        acc = fmaf(dT[(int64_t)b * E + o], P[L.oW2 + (int64_t)h * E + o], acc);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1)
+        acc += __shfl_xor_sync(FULL, acc, o);
+    if (lane == 0)
+        dZ[pair] = H[pair] > 0.f ? acc : 0.f;
+}
+
+// G[r][c] = (add: +=) sum_b A[b][r] D[b][c] for r < rows (times the input scale when scale is set),
+// row r = rows the sums of D, b ascending: W1 | b1 or W2 | b2 from G on.
+// COLS columns of THREADS / COLS rows a block
+template <int COLS, int THREADS>
+__global__ void few_gw_kernel(const float *__restrict__ A, int rows,
+                              const float *__restrict__ scale, const float *__restrict__ D,
+                              int cols, int B, float *__restrict__ G, bool add) {
+    const int c = blockIdx.x * COLS + threadIdx.x % COLS;
+    const int r = blockIdx.y * (THREADS / COLS) + threadIdx.x / COLS;
+    if (c >= cols || r > rows)
+        return;
+    const float s = scale != nullptr ? *scale : 1.f;
+    const float *pd = D + c;
+    float acc = 0.f;
+    if (r < rows) {
+        const float *pa = A + r;
+#pragma unroll 8
+        for (int b = 0; b < B; ++b)
+            acc = fmaf(s * pa[(int64_t)b * rows], pd[(int64_t)b * cols], acc);
+    } else {
+#pragma unroll 8
+        for (int b = 0; b < B; ++b)
+            acc += pd[(int64_t)b * cols];
+    }
+    float *g = G + (int64_t)r * cols + c;
+    *g = add ? *g + acc : acc;
 }
 
 // Adam (beta1 0.9, beta2 0.999) on every parameter but the input scale (index 0)
@@ -807,7 +915,7 @@ int entry_train_chunk(int64_t n, int d, int E) {
 }
 
 // Working memory of one chunk of B samples: H, dZ [B][64], T [B][E], the slices' partial
-// sums of (W1 | b1) and (W2 | b2) and the losses [ceil(B/8)].
+// sums of (W1 | b1) and (W2 | b2), and the losses [ceil(B/8)].
 size_t entry_train_chunk_bytes(int B, int d, int E) {
     const size_t slices = ((size_t)B + SLICE - 1) / SLICE;
     return sizeof(float) * ((size_t)B * EH * 2 + (size_t)B * E + ((size_t)B + 7) / 8 +
@@ -815,11 +923,19 @@ size_t entry_train_chunk_bytes(int B, int d, int E) {
            1024;
 }
 
-// Adds the gradient of the loss over samples [0, n) (divided by `total`) to G and the loss
-// to *loss, in chunks of B samples.
-cudaError_t entry_grad_accumulate(const float *P, int d, int E, const float *X,
-                                  const int32_t *y, int64_t n, int64_t total, int B, float *G,
-                                  float *loss, void *work, cudaStream_t s) {
+// Which kernel takes dZ of nb samples: the warps cost about max(13, 4 + E / 44) ns a sample,
+// the tiles 5.6 us + 56 ns a cell whatever the samples (up to a tile for each SM).  Measured,
+// warps | tiles: 512 samples of 64 cells 9.0 | 9.2 us, 1,024 of 256 14.9 | 18.8, 2,048 of 256
+// 25.9 | 19.4, 2,048 of 1,024 57 | 60.
+static bool tiled_dz(int64_t nb, int64_t E) {
+    return nb * (184 + E > 576 ? 184 + E : 576) >= 2450 * (100 + E);
+}
+
+// The gradient of the loss over samples [0, n), n >= 1 (divided by `total`), into G and the
+// loss into *loss, in chunks of B samples; the first chunk sets them (clearing them before
+// would be one or two launches more).
+cudaError_t entry_grad(const float *P, int d, int E, const float *X, const int32_t *y, int64_t n,
+                       int64_t total, int B, float *G, float *loss, void *work, cudaStream_t s) {
     const EntryLayout L = entry_layout(d, E);
     const int64_t n1 = (int64_t)(d + 1) * EH, n2 = (int64_t)(EH + 1) * E;
     float *H = reinterpret_cast<float *>(work);
@@ -836,19 +952,40 @@ cudaError_t entry_grad_accumulate(const float *P, int d, int E, const float *X,
         const float *Xb = X + b0 * d;
         const unsigned bt = (unsigned)((nb + GT - 1) / GT);
         const unsigned sl = (unsigned)((nb + SLICE - 1) / SLICE);
-        train_hidden_kernel<<<bt, 256, 0, s>>>(P, Xb, nb, d, H, L);
-        train_out_kernel<<<dim3(bt, et), 256, 0, s>>>(P, H, nb, E, T, L);
-        train_softmax_kernel<<<(nb + 7) / 8, 256, 0, s>>>(T, y + b0, nb, E, inv, losses);
-        train_gw_kernel<<<dim3(et, EH / GT, sl), 256, 0, s>>>(H, EH, nullptr, T, E, nb,
-                                                                    part2);
-        if (E <= 256)
+        const unsigned pairs = (unsigned)(((int64_t)nb * EH + 7) / 8);
+        const bool few = nb <= FEW && (int64_t)nb * E <= FEW_OUT;
+        const int nlosses = (nb + 7) / 8;
+        const bool add = b0 > 0;
+        if (nb <= FEW_HIDDEN)
+            few_hidden_kernel<<<(nb + 3) / 4, 256, 0, s>>>(P, Xb, nb, d, H, L);
+        else
+            train_hidden_kernel<<<bt, 256, 0, s>>>(P, Xb, nb, d, H, L);
+        if (few)
+            few_out_kernel<<<dim3((E + 127) / 128, nb), 128, 0, s>>>(P, H, E, T, L);
+        else
+            train_out_kernel<<<dim3(bt, et), 256, 0, s>>>(P, H, nb, E, T, L);
+        train_softmax_kernel<<<nlosses, 256, 0, s>>>(T, y + b0, nb, E, inv, losses);
+        if (few)
+            few_gw_kernel<128, 128><<<dim3((E + 127) / 128, EH + 1), 128, 0, s>>>(
+                H, EH, nullptr, T, E, nb, G + L.oW2, add);
+        else
+            train_gw_kernel<<<dim3(et, EH / GT, sl), 256, 0, s>>>(H, EH, nullptr, T, E, nb, part2);
+        if (!tiled_dz(nb, E))
+            few_dz_kernel<<<pairs, 256, 0, s>>>(P, H, T, nb, E, dZ, L, losses, nlosses,
+                                                few ? loss : nullptr, G, add);
+        else if (E <= 256)
             train_dz_kernel<1><<<bt, 256, 0, s>>>(P, H, T, nb, E, dZ, L);
         else
             train_dz_kernel<2><<<bt, 256, 0, s>>>(P, H, T, nb, E, dZ, L);
-        train_gw_kernel<<<dim3(1, (unsigned)((d + GT - 1) / GT), sl), 256, 0, s>>>(Xb, d, P, dZ, EH,
-                                                                              nb, part1);
-        grad_reduce_kernel<<<grid_for(n1 + n2, 32), 256, 0, s>>>(part1, n1, part2, n2, (int)sl, G,
-                                                                 losses, (nb + 7) / 8, loss);
+        if (few) {
+            few_gw_kernel<64, 256><<<dim3(1, (unsigned)(d + 4) / 4), 256, 0, s>>>(
+                Xb, d, P, dZ, EH, nb, G + L.oW1, add);
+        } else {
+            train_gw_kernel<<<dim3(1, (unsigned)((d + GT - 1) / GT), sl), 256, 0, s>>>(
+                Xb, d, P, dZ, EH, nb, part1);
+            grad_reduce_kernel<<<grid_for(n1 + n2, 32) + 1, 256, 0, s>>>(
+                part1, n1, part2, n2, (int)sl, G, losses, nlosses, loss, add);
+        }
         if ((e = cudaGetLastError()) != cudaSuccess)
             return e;
     }

@@ -948,15 +948,15 @@ nhq_status nhq_entry_grad(const float *params, int32_t d, int32_t E, const float
         return fail(NHQ_ERR_ARG, "the entry-model calls take device pointers");
     cudaStream_t s = as_stream(stream);
     const int64_t np = entry_param_count(d, E);
-    CK(cudaMemsetAsync(grad, 0, sizeof(float) * (size_t)np, s));
-    CK(cudaMemsetAsync(loss, 0, sizeof(float), s));
-    if (n == 0)
+    if (n == 0) {
+        CK(cudaMemsetAsync(grad, 0, sizeof(float) * (size_t)np, s));
+        CK(cudaMemsetAsync(loss, 0, sizeof(float), s));
         return NHQ_OK;
+    }
     const int B = entry_train_chunk(n, d, E);
     void *work = nullptr;
     CK(cudaMallocAsync(&work, entry_train_chunk_bytes(B, d, E), s));
-    cudaError_t e = entry_grad_accumulate(params, d, E, queries, labels, n, n, B, grad, loss,
-                                          work, s);
+    cudaError_t e = entry_grad(params, d, E, queries, labels, n, n, B, grad, loss, work, s);
     cudaFreeAsync(work, s);
     if (e != cudaSuccess)
         return fail_cuda(e, "nhq_entry_grad");
@@ -987,10 +987,7 @@ nhq_status nhq_entry_train(float *params, int32_t d, int32_t E, const float *que
     for (int ep = 0; ep < epochs && e == cudaSuccess; ++ep) {
         for (int64_t b = 0; b < n && e == cudaSuccess; b += batch) {
             const int64_t nb = n - b < batch ? n - b : batch;
-            e = cudaMemsetAsync(g, 0, sizeof(float) * (size_t)(np + 1), s);
-            if (e == cudaSuccess)
-                e = entry_grad_accumulate(params, d, E, queries + b * d, labels + b, nb, nb, B,
-                                          g, loss, work, s);
+            e = entry_grad(params, d, E, queries + b * d, labels + b, nb, nb, B, g, loss, work, s);
             ++t;
             const float c1 = 1.f / (1.f - powf(0.9f, (float)t));
             const float c2 = 1.f / (1.f - powf(0.999f, (float)t));

@@ -438,9 +438,8 @@ cudaError_t launch_entry_labels(const uint32_t *ids, int k, int64_t n, const uin
                                 int64_t N, int32_t *labels, cudaStream_t s);
 int entry_train_chunk(int64_t n, int d, int E);
 size_t entry_train_chunk_bytes(int B, int d, int E);
-cudaError_t entry_grad_accumulate(const float *P, int d, int E, const float *X,
-                                  const int32_t *y, int64_t n, int64_t total, int B, float *G,
-                                  float *loss, void *work, cudaStream_t s);
+cudaError_t entry_grad(const float *P, int d, int E, const float *X, const int32_t *y, int64_t n,
+                       int64_t total, int B, float *G, float *loss, void *work, cudaStream_t s);
 cudaError_t launch_entry_adam(float *p, const float *g, float *m, float *v, int64_t n, float lr,
                               float c1, float c2, cudaStream_t s);
 // acc[0] = sum over queries with a valid truth entry of |ids & truth| / valid, acc[1] = their count

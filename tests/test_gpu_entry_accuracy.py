@@ -71,3 +71,23 @@ def test_hidden_gradient_rounds_no_more_than_lane_sums(nhq, n, E):
             X = dev((rng.standard_normal((n, d)) * 0.1).astype(np.float32))
     rms = [float(np.sqrt(np.mean(np.square(e)))) for e in (ours, lanes)]
     assert rms[0] <= 1.15 * rms[1], rms
+
+
+# the kernels for few samples and their limits (128 samples, 2^18 outputs), and two chunks of
+# a batch whose second one is small (2,560 + 40 samples) or not (2,560 + 200)
+@pytest.mark.parametrize("d,E,n", [(3, 5, 2), (40, 300, 128), (40, 300, 129), (16, 4096, 64),
+                                   (16, 4096, 65), (16, 4096, 2600), (16, 4096, 2760)])
+def test_gradient_of_few_samples_and_of_several_chunks(nhq, d, E, n):
+    rng = np.random.default_rng(d + E + n)
+    p = (rng.standard_normal(mlp.entry_size(d, E)) * 0.2).astype(np.float32)
+    p[0] = 0.5 / np.sqrt(d)
+    Q = rng.standard_normal((n, d)).astype(np.float32)
+    y = rng.integers(0, E, n).astype(np.int32)
+    grad = torch.full((p.size,), float("nan"), dtype=torch.float32, device="cuda:0")
+    loss = torch.full((1,), float("nan"), dtype=torch.float32, device="cuda:0")
+    nhq.nhq_entry_grad(dev(p), E, dev(Q), dev(y), grad, loss)
+    torch.cuda.synchronize()
+    lw, gw = mlp.entry_loss_and_grad(p.astype(np.float64), Q, y, d, E)
+    # f32 sums of at most 2,760 terms: relative 1e-4 of each sum's largest terms
+    assert abs(loss.item() - lw) <= 1e-4 * abs(lw)
+    assert np.allclose(grad.cpu().numpy(), gw, rtol=1e-3, atol=1e-5 * np.abs(gw).max())
