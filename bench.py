@@ -191,6 +191,33 @@ def recorded_traffic(ef, h, vec, seed_mode, n, nq, learned):
     return float(rec["dram_bytes_per_launch"]) if same else None
 
 
+def split_details(line):
+    """(result line, details): sweeps and the long notes of the baselines stay out of the
+    result line, so that it is whole in the last 2,500 characters of the output (a line of
+    60 KB lost its start wherever only the end of the output is kept).  Floats carry seven
+    digits."""
+    def short(x):
+        if isinstance(x, float):
+            return float(f"{x:.7g}")
+        if isinstance(x, dict):
+            return {k: short(v) for k, v in x.items()}
+        return [short(v) for v in x] if isinstance(x, (list, tuple)) else x
+
+    out, details = dict(line), {}
+    for key in ("sweep", "learned", "plain_f32", "brute_force", "cpu_baseline"):
+        details[key] = out.pop(key, None)
+    bf, cpu = details["brute_force"], details["cpu_baseline"]
+    if bf:
+        out["brute_force"] = {k: bf[k] for k in ("bound", "ms", "achieved", "peak", "unit",
+                                                 "frac") if k in bf}
+    if cpu:
+        out["cpu_baseline"] = {k: cpu[k] for k in ("value", "unit", "cores", "kind") if k in cpu}
+        for name in ("all_cores", "search"):
+            if name in cpu:
+                out["cpu_baseline"][name] = cpu[name].get("value")
+    return short(out), details
+
+
 def fp32_simt_peak(dev):
     """Measured FP32 throughput of the SIMT units: cuBLAS SGEMM with TF32 off (8192^3),
     TFLOP/s; the denominator of the brute force's ALU roofline."""
@@ -1829,6 +1856,8 @@ def main():
                 w, a, nbr, ef, a.seed_mode, ids.cpu().numpy(), 4 * a.cpu_sample, h, vec)
     ix.close()
     if rank == 0:
+        line, details = split_details(line)
+        print(json.dumps({"details": details}), file=sys.stderr, flush=True)
         print(json.dumps(line), flush=True)
     if dist is not None:
         dist.destroy_process_group()
