@@ -21,13 +21,15 @@
 // through the full scan afterwards, counted on the device; a long run that is going to fail
 // is given up early.
 //
-// What bounds it: the full scan the FP32 pipe and the issue slots around it.  Candidate
-// sets of 60,000 objects (d = 96, K = 64, proportional weights) take 41.2 ms, half the FP32
+// What bounds it: 64 % of the issue slots and 56 % of the FMA pipe's cycles are used, by 21
+// warps an SM that wait for shared memory, barriers and fixed latencies about equally (80
+// registers, 8 bytes spilled, for three CTAs an SM).  Candidate
+// sets of 60,000 objects (d = 96, K = 64, proportional weights) take 40.0 ms, half the FP32
 // rate of a difference and an fma per dimension; before (no staging ahead, every pair's
 // Gamma with its division, records inserted one by one) 55.5 ms.  2,003 queries, k = 100,
-// over 300,007 objects: 10.6 ms, before 16.4 ms.  The runs do a hundredth of the pairs: the
-// filter truth of 10,000 queries over a million objects (600 tuples) 1.67 ms, before 206 ms;
-// eight queries under constant weights 62 us, before 5,560 us.
+// over 300,007 objects: 9.8 ms, before 16.4 ms.  The runs do a hundredth of the pairs: the
+// filter truth of 10,000 queries over a million objects (600 tuples) 1.58 ms, before 206 ms;
+// eight queries under constant weights 59 us, before 5,560 us.
 #include <cmath>
 #include <cstdio>
 #include <mutex>
@@ -850,7 +852,8 @@ cudaError_t launch_scan(const TopkArgs &a, const ScanQueries &sq, int sm_count, 
 
 // Which tile a full scan takes, and its slices.  Up to 8 queries the scan is bound by
 // reading the objects, and tiles of 4 queries leave the fewest idle pairs; beyond, tiles of
-// 32.  (Tiles of 64 queries, 4 x 8 pairs a thread, read shared memory less per pair but fit
+// 32.  300,000 objects, d = 96, k = 10, tiles of 4 | 32: 4 queries 113 | 243 us, 8 121 | 250,
+// 16 155 | 259, 32 230 | 268, so the line could lie higher.  (Tiles of 64 queries, 4 x 8 pairs a thread, read shared memory less per pair but fit
 // two CTAs an SM: 53.2 ms against 44.8 ms for the candidate sets of 60,000 objects.)
 struct ScanPlan {
     int shape;  // queries per tile: 4 or 32
@@ -1018,7 +1021,9 @@ cudaError_t launch_topk_runs(const TopkArgs &args, const uint8_t *codes,
     p.codes = codes;
     if (codes != nullptr)
         a.qattr = p.words;
-    // Few queries hardly share tuples: tiles of 4.
+    // Few queries hardly share tuples: tiles of 4.  A million objects of 600 even tuples, d =
+    // 128, k = 10, tiles of 4 | 32: 8 queries 44 | 73 us, 64 54 | 85, 256 115 | 209, so the line
+    // could lie higher.
     const bool few = a.nq <= 64;
     p.tq = few ? Narrow::TQ : Mid::TQ;
     p.slice = run_slice_length(a.nq);

@@ -13,7 +13,8 @@
 // depend on this order.
 //
 // One CTA owns 128 rows and sweeps all column tiles of 128, starting at its
-// own (diagonal) tile so that each row first meets the objects of its own tuple
+// own (diagonal) tile, or under constant weights the one before it where its first tuple's
+// run is cut, so that each row first meets the objects of its own tuple
 // (concurrent CTAs then read a sliding window of neighbouring tiles from L2):
 //   warp 0              scheduler + TMA: decides for each tile whether any row
 //                       can still take a record from it (skipped tiles are never

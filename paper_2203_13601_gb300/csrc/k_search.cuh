@@ -311,8 +311,10 @@ __device__ __forceinline__ unsigned long long filter_key(unsigned long long c,
 // that no candidate takes receives the old record as many places below it as candidates
 // precede it.  Chunks go from the top down, each read before it is written.
 // A chunk costs about 20 instructions whatever the number of candidates (it was 15 plus 6
-// for each of up to 8, or a sort and a binary search per record beyond): 1,000 queries at
-// ef 100 on 10,000 objects 428 -> 391 us, 10,000 at ef 24 on a million 472 -> 451 us.
+// for each of up to 8, or a sort and a binary search per record beyond): 10,000 queries at
+// ef 24 on a million objects 472 -> 451 us, one query at ef 1,000 3.18 -> 2.70 ms; 1,000
+// queries at ef 100 on 10,000 objects 428 -> 391 us on one machine, inside the spread of 8 %
+// on another.
 __device__ void merge_round(unsigned long long *pool, int &n, int ef, unsigned long long c,
                             unsigned long long *cand32, int lane) {
     if (c != kInfKey && n == ef && c > (pool[ef - 1] & ~1ull))

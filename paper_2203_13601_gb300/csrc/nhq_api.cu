@@ -438,8 +438,11 @@ static nhq_status exact_room(nhq_index *ix, size_t need, bool capturing) {
 
 // Whether an exact top-k over all objects takes the tuple runs of the attribute order.
 // They cost four to seven launches against the scan's three, so a scan of less than 2^26
-// pair dimensions (under 20 us) is left alone; where the order does not exist yet, sorting
-// the words and allocating it (about 0.3 ms once) has to pay in this very call.  A capture
+// pair dimensions is left alone (runs | scan: 100 queries over 2,000 objects, d = 32, constant
+// weights, 145 | 125 us, over 10,000, 2^25, 46 | 125: the line could lie lower); where the
+// order does not exist yet, sorting the words and allocating it has to pay in this very call
+// (8 queries over 50,000 objects, d = 128, 167 | 107 us, 100 over 40,000, d = 64, 2^28,
+// 194 | 181, 1,000 over 10,000, 2^29.3, 175 | 208).  A capture
 // takes the order that is there: one made in it would be sorted at its launches only.
 static bool take_runs(const nhq_index *ix, const TopkArgs &a, bool capturing) {
     if (!topk_runs_apply(a))

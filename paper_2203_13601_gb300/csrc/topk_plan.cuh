@@ -51,7 +51,9 @@ constexpr int MAX_SLICES = 128;
 // Objects per slice of a tuple's run.  Few queries hardly share tuples: short slices, so
 // that one query's run fills the chip (9,000 objects on average at a million and 600
 // tuples: 36 slices of 256).  Larger batches fill it with tiles of 32 queries and pay for
-// slices in lists.
+// slices in lists.  A million objects of 600 even tuples, d = 128, k = 10: 8 queries 37 us
+// in slices of 128, 44 of 256, 68 of 1,024; 64 queries 56, 54 and 85; 2,000 queries 521 us of
+// 256, 500 of 1,024, 538 of 2,048; 10,000 queries 612, 567 and 577.
 __host__ __device__ inline int run_slice_length(int64_t nq) {
     return nq <= 64 ? 256 : nq <= 2048 ? 1024 : 2048;
 }
