@@ -45,6 +45,7 @@ constexpr int DC = 32;      // dimensions per staged chunk
 constexpr int DS = DC + 4;  // staged row stride: 16-byte aligned rows, read as float4
 constexpr int NT = 256;     // threads per CTA
 constexpr uint32_t PROBE = 512;  // objects (k <= 256) after which a long run is judged
+constexpr uint32_t GIVEN_UP = 0x80000000u;  // a run's length is below 2^31
 constexpr unsigned FULL = 0xFFFFFFFFu;
 constexpr float INF = __builtin_huge_valf();
 constexpr unsigned long long NO_RECORD = (0x7F800000ull << 32) | kNone;  // (inf, none)
@@ -565,10 +566,9 @@ struct RunGroup {
 };
 struct RunPlan {
     RunHeader *hdr;
-    uint32_t *failed;  // [nq] queries that a long run was given up for (constant weights)
     uint32_t *key, *tcnt, *tgroup;  // [T] run start + 1, queries, group
     uint32_t tmask;
-    uint32_t *lo, *len, *home, *rank;  // [nq]
+    uint32_t *lo, *len, *home, *rank;  // [nq]; len with GIVEN_UP where the run was given up
     uint32_t *slot;                    // [nq] queries in group order
     RunGroup *group;                   // [nq]
     uint32_t *left;                    // [nq] queries for the full scan
@@ -580,6 +580,7 @@ struct RunPlan {
     uint32_t *words;
     int tq, slice;  // queries per unit, objects per slice aimed at
     int busy;       // tiles of queries that fill the chip
+    bool scarce;    // the runs may ask for more list rows than there are
 };
 
 __device__ __forceinline__ int64_t lower_bound_word(const uint32_t *a, int64_t n, uint32_t x) {
@@ -612,8 +613,10 @@ __device__ __forceinline__ unsigned plan_lookup(const TopkArgs &a, const RunPlan
         return 0;
     uint32_t s = table_slot((uint32_t)l, p.tmask);
     for (uint32_t probe = 0; probe <= p.tmask; ++probe) {  // half empty: ends
-        // a key stays once it is set, so only an empty slot needs the exchange
-        uint32_t x = *reinterpret_cast<const volatile uint32_t *>(&p.key[s]);
+        // a key stays once it is set, so only an empty slot needs the exchange; few queries
+        // hardly meet one another's, and save the read's latency
+        uint32_t x =
+            a.nq <= 64 ? 0u : *reinterpret_cast<const volatile uint32_t *>(&p.key[s]);
         if (x == 0u)
             x = atomicCAS(&p.key[s], 0u, (uint32_t)l + 1u);
         if (x == 0u || x == (uint32_t)l + 1u)
@@ -628,6 +631,8 @@ __device__ __forceinline__ unsigned plan_lookup(const TopkArgs &a, const RunPlan
 
 // adds up what a warp's queries ask for
 __device__ __forceinline__ void plan_ask(const RunPlan &p, unsigned mine) {
+    if (!p.scarce)
+        return;
     const unsigned sum = __reduce_add_sync(FULL, mine);
     if ((threadIdx.x & 31) == 0 && sum > 0)
         atomicAdd(&p.hdr->asked, (unsigned long long)sum);
@@ -644,7 +649,9 @@ __device__ __forceinline__ void plan_group(const RunPlan &p, int64_t q) {
     const int64_t tiles = (g.cnt + p.tq - 1) / p.tq;
     const int64_t s =
         granted_slices(run_slices(g.len, p.slice), tiles,
-                       *reinterpret_cast<const volatile unsigned long long *>(&p.hdr->asked),
+                       p.scarce ? *reinterpret_cast<const volatile unsigned long long *>(
+                                      &p.hdr->asked)
+                                : 0ull,
                        p.rows, p.busy);
     g.lbase = s > 1 ? atomicAdd(&p.hdr->list_rows, (unsigned long long)g.cnt * s) : 0;
     g.slices = (int)s;
@@ -685,8 +692,6 @@ __global__ void __launch_bounds__(1024) run_plan_kernel(TopkArgs a, RunPlan p) {
         *p.hdr = RunHeader{};
     for (uint32_t t = threadIdx.x; t <= p.tmask; t += blockDim.x)
         p.key[t] = p.tcnt[t] = 0u;
-    for (int64_t q = threadIdx.x; q < a.nq; q += blockDim.x)
-        p.failed[q] = 0u;
     __syncthreads();
     unsigned asked = 0;
     for (int64_t q = threadIdx.x; q < a.nq; q += blockDim.x)
@@ -744,7 +749,7 @@ __global__ void __launch_bounds__(NT, T::CTAS) run_kernel(TopkArgs a, RunPlan p)
             sm.q[r] = q;
             wanted = wanted ||
                      (q != kNone &&
-                      *reinterpret_cast<const volatile uint32_t *>(p.failed + q) == 0u);
+                      (*reinterpret_cast<const volatile uint32_t *>(p.len + q) & GIVEN_UP) == 0u);
         }
         if (!__syncthreads_or(wanted))
             continue;  // another slice has given up for all of them
@@ -756,7 +761,7 @@ __global__ void __launch_bounds__(NT, T::CTAS) run_kernel(TopkArgs a, RunPlan p)
         if (!scan_objects<T, true>(a, sm, lists, (uint32_t)begin, (uint32_t)end, p.id_sorted,
                                    nullptr, until)) {
             for (int r = tid; r < T::TQ; r += NT)
-                if (sm.q[r] != kNone && atomicExch(p.failed + sm.q[r], 1u) == 0u)
+                if (sm.q[r] != kNone && (atomicOr(p.len + sm.q[r], GIVEN_UP) & GIVEN_UP) == 0u)
                     p.left[atomicAdd(&p.hdr->left, 1u)] = sm.q[r];
             continue;
         }
@@ -792,13 +797,16 @@ __global__ void run_merge_kernel(TopkArgs a, RunPlan p) {
     for (int64_t q = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); q < a.nq;
          q += (int64_t)gridDim.x * (blockDim.x >> 5)) {
         float last = INF;
-        if (p.len[q] == 0) {
+        const uint32_t len = p.len[q];
+        if (len & GIVEN_UP)
+            continue;
+        if (len == 0) {
             for (int e = lane; e < a.k; e += 32)
                 write_record(a, q, e, INF, kNone);
         } else {
             const RunGroup &g = p.group[p.tgroup[p.home[q]]];
             const int S = g.slices;
-            if (S == 1 || (a.w.mode != NHQ_W_FILTER && p.failed[q] != 0u))
+            if (S == 1)
                 continue;
             const int64_t o = ((int64_t)g.lbase + (int64_t)p.rank[q] * S) * a.k;
             merge_lists(p.part_id + o, p.part_g + o, S, a.k, lane,
@@ -808,7 +816,7 @@ __global__ void run_merge_kernel(TopkArgs a, RunPlan p) {
                             last = gm;
                         });
         }
-        if (lane == 0 && a.w.mode != NHQ_W_FILTER && p.len[q] < a.N && !(last < fusion_gamma(0.f, 1, a.w)))
+        if (lane == 0 && a.w.mode != NHQ_W_FILTER && len < a.N && !(last < fusion_gamma(0.f, 1, a.w)))
             p.left[atomicAdd(&p.hdr->left, 1u)] = (uint32_t)q;
     }
 }
@@ -928,7 +936,7 @@ cudaError_t launch_topk(const TopkArgs &a, void *scratch, size_t scratch_bytes, 
 namespace {
 
 struct RunLayout {
-    size_t failed, table, words, query, slot, group, left, part, kth, scan, bytes;
+    size_t table, words, query, slot, group, left, part, kth, scan, bytes;
     uint32_t tmask;
     int64_t rows, srows;
 };
@@ -949,7 +957,6 @@ RunLayout run_layout(const TopkArgs &a, int sm_count) {
         off += (bytes + 255) & ~(size_t)255;
         return at;
     };
-    L.failed = take(sizeof(uint32_t) * (size_t)a.nq);
     L.table = take(3 * sizeof(uint32_t) * (size_t)T);
     L.words = take(sizeof(uint32_t) * (size_t)a.nq);
     L.query = take(4 * sizeof(uint32_t) * (size_t)a.nq);
@@ -1000,7 +1007,6 @@ cudaError_t launch_topk_runs(const TopkArgs &args, const uint8_t *codes,
     RunPlan p;
     const size_t T = (size_t)L.tmask + 1;
     p.hdr = reinterpret_cast<RunHeader *>(base);
-    p.failed = reinterpret_cast<uint32_t *>(base + L.failed);
     p.key = reinterpret_cast<uint32_t *>(base + L.table);
     p.tcnt = p.key + T;
     p.tgroup = p.tcnt + T;
@@ -1029,6 +1035,7 @@ cudaError_t launch_topk_runs(const TopkArgs &args, const uint8_t *codes,
     p.slice = run_slice_length(a.nq);
     const int ctas = few ? resident_ctas<Narrow>(a.k, sm_count) : resident_ctas<Mid>(a.k, sm_count);
     p.busy = 2 * ctas;
+    p.scarce = a.nq * run_slices(a.N, p.slice) > L.rows && L.rows > 0;
     cudaError_t e;
     if (a.nq <= 2048) {
         run_plan_kernel<<<1, a.nq <= 256 ? 256 : 1024, 0, s>>>(a, p);
