@@ -329,8 +329,9 @@ constexpr int SLICE = 128;
 // Up to FEW samples and FEW_OUT outputs a step takes kernels with a thread to an output, and
 // up to FEW_HIDDEN samples that for H.  Steps at d = 128, on them | on the tiles: 32 samples
 // 39.6 | 45.7 us (64 and 256 cells) and 57.5 | 66.7 us (4,096), 128 samples 53.9 | 57.9 and
-// 84.2 | 83.0, 200 samples 64.4 | 59.0 and 107 | 92; H alone takes 2 us off at 1,024 and
-// 2,048 samples (14 at d = 960) and adds 2 to 28 at 4,096.
+// 84.2 | 83.0, 200 samples 64.4 | 59.0 and 107 | 92 (each with 4 us of clearing that are gone
+// now); H alone takes 2 us off at 1,024 and 2,048 samples (14 at d = 960) and adds 2 to 28 at
+// 4,096.
 constexpr int FEW = 128, FEW_HIDDEN = 2048;
 constexpr int64_t FEW_OUT = 1 << 18;  // samples x cells
 
@@ -341,8 +342,9 @@ constexpr int64_t FEW_OUT = 1 << 18;  // samples x cells
 // chunk) as another and the chunks as a third; 2 also eight chunks apart from the rest.
 // One chain over the E cells of a gradient had up to five times the error of 32 strided
 // chains and a tree, which summed them before; 1 has it times 1.1 up to E = 256, 2 times 0.5
-// from 1,024 on (1 would have 1.25 at 4,096).  At E = 256 a step takes 133.6 us with 0 and
-// 1, 135.7 us with 2 or with Kahan's compensation per chunk.
+// from 1,024 on (1 would have 1.25 at 4,096).  At E = 256 a step took 133.6 us with 0 and
+// 1, 135.7 us with 2 or with Kahan's compensation per chunk (each 4 us less since the gradient
+// and the loss need no clearing).
 template <bool AK, bool BK, int LEVELS = 0, class LA, class LB>
 __device__ __forceinline__ void tile_product(float acc[4][4], int64_t k0, int64_t k1, LA la, LB lb,
                                              float (*As)[GP], float (*Bs)[GP],
